@@ -220,6 +220,22 @@ __device__ __forceinline__ void pdl_enter()
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Preferred shared-memory carveout (percent; -1: the driver's choice per kernel) of
+// the launches a host thread makes while a LaunchScope lives.  An SM runs one split
+// of its storage between shared memory and L1 at a time, so a kernel that asks for
+// another split than its predecessor's cannot start on an SM before that has
+// drained, and the early launch above is lost.  In a small system, whose kernels
+// last 5 to 30 us, one split for all kernels of a step is worth more than the split
+// each would get (see step_carveout).
+struct LaunchScope {
+    static inline thread_local int carveout = -1;
+    int saved;
+    explicit LaunchScope(int percent) : saved(carveout) { carveout = percent; }
+    ~LaunchScope() { carveout = saved; }
+    LaunchScope(const LaunchScope&) = delete;
+    LaunchScope& operator=(const LaunchScope&) = delete;
+};
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl_smem(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                    cudaStream_t st, Args&&... args)
@@ -229,11 +245,16 @@ inline cudaError_t launch_pdl_smem(void (*kern)(KArgs...), dim3 grid, dim3 block
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    if (LaunchScope::carveout >= 0) {
+        attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        attr[1].val.sharedMemCarveout = (unsigned)LaunchScope::carveout;
+        cfg.numAttrs = 2;
+    }
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
