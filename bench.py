@@ -645,16 +645,15 @@ def run_ours(args):
         import numpy as np
         xs, _, ts, _ = s.state()
         ws = w if args.workload == "batch" else [w]
-        split_density = (tuned and tuned["chosen"] == "nlist-thread") or \
-            args.kernels == "nlist-thread"
+        split_density = args.kernels != "scan"
         off = 0
         cand = 0
         for wr in ws:
             nr = wr.n if args.workload == "batch" else n
             p = wr.params
             ncell = [max(1, int(math.floor(p.box[k] / p.rc))) for k in range(3)]
-            # the thread-per-particle pass of a single system with frozen
-            # particles runs the frozen split
+            # the list pass of a single system with frozen particles runs the
+            # frozen split
             fz = None
             if args.workload != "batch" and p.frozen_types and split_density:
                 fz = np.isin(ts[off:off + nr], np.array(p.frozen_types))
@@ -716,8 +715,7 @@ def run_ours(args):
         # lists: 4 B per directed partner; FP32 tiles 16 B (FP64 32 B)
         tile = 16 if prec == 1 else 32
         npart = pairs / max(n, 1)
-        dens_name = "k_density_cell" if (tuned and tuned["chosen"] == "nlist") or \
-            args.kernels == "nlist" else "k_density_nl"
+        dens_name = "k_density_nl"
 
         def entry(name, work, ms_k, bytes_pp, what):
             if ms_k <= 0:
@@ -845,8 +843,7 @@ def main():
     ap.add_argument("--nrep", type=int, default=256, help="replicas of the batch workload")
     ap.add_argument("--kernels", choices=("auto", "nlist", "nlist-thread", "scan"), default="auto")
     ap.add_argument("--density-shape", type=int, choices=(0, 1), default=None,
-                    help="code shape of the thread-per-particle density kernel when "
-                         "--kernels is not auto")
+                    help="MDPD_OPT_DENSITY_SHAPE when --kernels is not auto (without effect)")
     ap.add_argument("--force-lanes", type=int, choices=(1, 2, 4), default=None,
                     help="lanes per particle of the force pass when --kernels is not auto")
     ap.add_argument("--profile-every", type=int, default=10,

@@ -245,18 +245,16 @@ int mdpd_pair_count(mdpd_handle* h, int64_t* pairs);
  *                      0: launch kernels one by one.
  *   MDPD_OPT_PROFILE   k > 0: record CUDA events around every kernel class of
  *                      the next steps (up to k steps); 0: off.
- *   MDPD_OPT_KERNELS   MDPD_KERNELS_NLIST (default): a warp-per-cell density
- *                      pass records each mobile particle's partners within r_c
- *                      and the force pass walks that list;
- *                      MDPD_KERNELS_NLIST_THREAD: the same with a
- *                      thread-per-particle density pass; MDPD_KERNELS_SCAN:
+ *   MDPD_OPT_KERNELS   MDPD_KERNELS_NLIST (default) and
+ *                      MDPD_KERNELS_NLIST_THREAD (the same): the density pass
+ *                      records each mobile particle's partners within r_c and
+ *                      the force pass walks that list; MDPD_KERNELS_SCAN:
  *                      both passes scan the 27 neighbour cells directly.
  *                      Same results up to FP summation order.
  *   MDPD_OPT_WALL_DENSITY  1: every density pass also accumulates the wall
  *                      density phi of each mobile particle (Sec. 3.2,
- *                      Algorithm 1 step 2; read with mdpd_get_wall_density);
- *                      the thread-per-particle density variant is used while
- *                      it is on.  0 (default): off.
+ *                      Algorithm 1 step 2; read with mdpd_get_wall_density).
+ *                      0 (default): off.
  *   MDPD_OPT_FORCE_LANES  1, 2 or 4 (default 1): lanes that share one
  *                      particle's partner list in the force pass (more warps
  *                      for small systems; the partner sums are combined in a
@@ -266,11 +264,8 @@ int mdpd_pair_count(mdpd_handle* h, int64_t* pairs);
  *   MDPD_OPT_PROFILE_EVERY  m >= 1: with MDPD_OPT_PROFILE on, record the events
  *                      on every m-th step only (default 1), which keeps their
  *                      cost out of most steps.
- *   MDPD_OPT_DENSITY_SHAPE  0 (default) or 1: code shape of the
- *                      thread-per-particle density kernel (candidate loop not
- *                      unrolled, or unrolled by two under a tighter register
- *                      budget).  Results are identical; only the speed
- *                      differs (mdpd_autotune picks the faster).
+ *   MDPD_OPT_DENSITY_SHAPE  0 (default) or 1: accepted and without effect (the
+ *                      density pass has one code shape).
  */
 enum { MDPD_OPT_GRAPH = 1, MDPD_OPT_PROFILE = 2, MDPD_OPT_KERNELS = 3,
        MDPD_OPT_PROFILE_EVERY = 4, MDPD_OPT_WALL_DENSITY = 5, MDPD_OPT_FORCE_LANES = 6,
@@ -379,15 +374,13 @@ int mdpd_window_vjp_dev(mdpd_handle* h, const double* xbar, const double* vbar,
                         const double* cvir, const double* rhobar, double* x0bar, double* v0bar,
                         double* theta_bar);
 
-/* Time the density-pass variants (MDPD_KERNELS_NLIST, MDPD_KERNELS_NLIST_THREAD
- * in both code shapes of MDPD_OPT_DENSITY_SHAPE) and then the force pass at 1,
- * 2 and 4 lanes per particle (MDPD_OPT_FORCE_LANES; 1 only on a batch) on the
- * current state, reps launches each, and keep the fastest of each.  The
- * trajectory is not advanced.  chosen (may be NULL, 3 ints) receives the
- * density variant, the lanes per particle and the code shape kept; ms (may be
- * NULL, 5 doubles) the mean time of each density variant in that order (the
- * thread variant's faster shape), then of the force pass at 1, 2, 4 lanes (-1:
- * not tried).  Synchronises. */
+/* Time the density pass and then the force pass at 1, 2 and 4 lanes per particle
+ * (MDPD_OPT_FORCE_LANES; 1 only on a batch) on the current state, reps launches
+ * each, and keep the fastest.  The trajectory is not advanced.  A handle on
+ * MDPD_KERNELS_SCAN changes to MDPD_KERNELS_NLIST.  chosen (may be NULL, 3
+ * ints) receives the density variant, the lanes per particle and 0; ms (may be
+ * NULL, 5 doubles) the mean time of the density pass (twice), then of the force
+ * pass at 1, 2, 4 lanes (-1: not tried).  Synchronises. */
 int mdpd_autotune(mdpd_handle* h, int32_t reps, int32_t* chosen, double* ms);
 
 /* Grid of the cell lattice (cells per axis) and the kernel launches one step

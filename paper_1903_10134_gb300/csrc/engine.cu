@@ -61,6 +61,8 @@ struct mdpd_handle {
     // cell-ordered compute arrays
     void* pos4 = nullptr;
     void* vel4 = nullptr;
+    void* fpos = nullptr;            // FP32 offsets beside FP64 ones
+    uint16_t* hpos = nullptr;        // FP16 positions of the density pass's filter
     void* rho = nullptr;
     uint32_t* cell_s = nullptr;
     // binning
@@ -94,7 +96,6 @@ struct mdpd_handle {
     bool want_phi = false;
     int kernels = MDPD_KERNELS_NLIST;
     int force_lpp = 1;               // lanes per particle of the force pass (single system)
-    int thread_shape = 0;            // code shape of the thread-per-particle density kernel
     bool walls_set = false;
     std::vector<int32_t> h_type;
     int64_t steps_host = 0;
@@ -119,11 +120,10 @@ struct mdpd_handle {
     std::vector<mdpd_params> rep_p;
     Rep* d_reps = nullptr;
     int4* d_chunks = nullptr;
-    int4* d_cchunks = nullptr;
     int2* d_wr = nullptr;
     double* obs_b = nullptr;
     Rep* d_reps_all = nullptr;       // the same records with list_all set (adjoint lists)
-    int nchunk = 0, ncchunk = 0;
+    int nchunk = 0;
 
     // adjoint: per-block parameter partials and per-replica sums, virial
     // weights, and a velocity-Verlet window's checkpoints (id order:
@@ -146,9 +146,7 @@ struct mdpd_handle {
         Batch b;
         b.reps = all && d_reps_all ? d_reps_all : d_reps;
         b.chunks = d_chunks;
-        b.cchunks = d_cchunks;
         b.nchunk = nchunk;
-        b.ncchunk = ncchunk;
         return b;
     }
 
@@ -214,6 +212,8 @@ void free_particles(mdpd_handle* h)
     }
     dfree(h->pos4);
     dfree(h->vel4);
+    dfree(h->fpos);
+    dfree(h->hpos);
     dfree(h->rho);
     dfree(h->cell_s);
     dfree(h->cellof);
@@ -248,6 +248,8 @@ int alloc_particles(mdpd_handle* h, int64_t cap)
     }
     if (!rc) rc = dalloc(h, &h->pos4, c * v4);
     if (!rc) rc = dalloc(h, &h->vel4, c * v4);
+    if (!rc && h->precision == 0) rc = dalloc(h, &h->fpos, c * sizeof(float4));
+    if (!rc) rc = dalloc(h, &h->hpos, hpos_words(c) * sizeof(uint16_t));
     if (!rc) rc = dalloc(h, &h->rho, c * tsz);
     if (!rc) rc = dalloc(h, &h->cell_s, c * sizeof(uint32_t));
     if (!rc) rc = dalloc(h, &h->cellof, c * sizeof(uint32_t));
@@ -286,6 +288,8 @@ void swap_particle_arrays(mdpd_handle* a, mdpd_handle* b)
     }
     std::swap(a->pos4, b->pos4);
     std::swap(a->vel4, b->vel4);
+    std::swap(a->fpos, b->fpos);
+    std::swap(a->hpos, b->hpos);
     std::swap(a->rho, b->rho);
     std::swap(a->cell_s, b->cell_s);
     std::swap(a->cellof, b->cellof);
@@ -497,11 +501,11 @@ void enqueue_bin(mdpd_handle* h, bool gather_a, bool kick = false)
     if (h->nrep)
         launch_rank_gather_batch(st, h->precision, h->cap, h->cellof, h->start, h->key, h->src,
                                  master(h, h->cur), master(h, 1 - h->cur), gather_a, h->batch(),
-                                 h->pos4, h->vel4, h->cell_s);
+                                 h->pos4, h->vel4, h->fpos, h->hpos, h->cell_s);
     else
         launch_rank_gather(st, h->precision, n, h->cap, h->cellof, h->start, h->key, h->src,
                            master(h, h->cur), master(h, 1 - h->cur), gather_a, h->geo, h->ph,
-                           h->pos4, h->vel4, h->cell_s);
+                           h->pos4, h->vel4, h->fpos, h->hpos, h->cell_s);
     h->cur = 1 - h->cur;
 }
 
@@ -514,12 +518,12 @@ int step_launches(const mdpd_handle* h)
     return 6 + scan_num_launches(h->geo.ncell) + (use_split(h) ? 1 : 0);
 }
 
-// The thread-per-particle density pass of a system with frozen particles
-// scans only mobile candidates for frozen homes (frozen split).
+// The density pass of a system with frozen particles scans for its mobile homes
+// only (frozen split).
 bool use_split(const mdpd_handle* h)
 {
     return !h->nrep && h->ph.frozen != 0 && !h->ph.list_all &&
-           (h->want_phi || h->kernels == MDPD_KERNELS_NLIST_THREAD);
+           (h->want_phi || h->kernels != MDPD_KERNELS_SCAN);
 }
 
 // The frozen-frozen density part, from the last binning (the frozen
@@ -527,8 +531,8 @@ bool use_split(const mdpd_handle* h)
 void ensure_ff(mdpd_handle* h)
 {
     if (!use_split(h) || !h->ff_dirty) return;
-    launch_density_nl(h->stream, h->precision, (int)h->n, h->cap, h->geo, h->ph, h->pos4,
-                      h->cell_s, h->start, h->rho, h->nl, h->nl_count, 2, h->facc, h->id[h->cur],
+    launch_density_nl(h->stream, h->precision, (int)h->n, h->cap, h->geo, h->ph, h->pos4, h->fpos,
+                      h->hpos, h->cell_s, h->start, h->rho, h->nl, h->nl_count, 2, h->facc, h->id[h->cur],
                       h->rho_ff);
     // the positions it was computed from (set_state keeps the part while the
     // frozen particles are loaded unmoved)
@@ -545,28 +549,18 @@ bool list_compact(const mdpd_handle* h) { return use_split(h) && h->force_lpp ==
 // a single system takes it from ph.list_all).
 void enqueue_density(mdpd_handle* h, bool all = false)
 {
-    const bool cell = h->kernels == MDPD_KERNELS_NLIST;
     if (h->nrep) {
-        if (cell)
-            launch_density_cell_batch(h->stream, h->precision, h->cap, h->batch(all), h->pos4,
-                                      h->start, h->rho, h->nl, h->nl_count);
-        else
-            launch_density_nl_batch(h->stream, h->precision, h->cap, h->batch(all), h->pos4,
-                                    h->cell_s, h->start, h->rho, h->nl, h->nl_count,
-                                    h->thread_shape);
+        launch_density_nl_batch(h->stream, h->precision, h->cap, h->batch(all), h->pos4, h->fpos,
+                                h->hpos, h->cell_s, h->start, h->rho, h->nl, h->nl_count);
         return;
     }
     h->ph.phi_out = h->want_phi ? h->phi : nullptr;
     h->ph.list_compact = list_compact(h) ? 1 : 0;
-    const int fs = use_split(h) ? 1 : 0;
-    if (h->want_phi || h->kernels == MDPD_KERNELS_NLIST_THREAD)
-        // (the wall density is accumulated by this variant only)
+    if (h->kernels != MDPD_KERNELS_SCAN || h->want_phi)
+        // (the wall density is accumulated by the list pass only)
         launch_density_nl(h->stream, h->precision, (int)h->n, h->cap, h->geo, h->ph, h->pos4,
-                          h->cell_s, h->start, h->rho, h->nl, h->nl_count, fs, h->facc,
-                          h->id[h->cur], h->rho_ff, h->thread_shape);
-    else if (cell)
-        launch_density_cell(h->stream, h->precision, h->geo.ncell, h->cap, h->geo, h->ph, h->pos4,
-                            h->start, h->rho, h->nl, h->nl_count);
+                          h->fpos, h->hpos, h->cell_s, h->start, h->rho, h->nl, h->nl_count,
+                          use_split(h) ? 1 : 0, h->facc, h->id[h->cur], h->rho_ff);
     else
         launch_density(h->stream, h->precision, (int)h->n, h->geo, h->ph, h->pos4, h->cell_s,
                        h->start, h->rho);
@@ -979,7 +973,7 @@ int create_batch(int32_t nrep, const mdpd_params* params, const int64_t* n, cons
     h->kernels = MDPD_KERNELS_NLIST;
     h->rep_p.assign(params, params + nrep);
     h->reps.resize((size_t)nrep);
-    std::vector<int4> chunks, cchunks;
+    std::vector<int4> chunks;
     std::vector<int2> wr((size_t)nrep);
     for (int r = 0; r < nrep; ++r) {
         Rep& R = h->reps[r];
@@ -998,19 +992,15 @@ int create_batch(int32_t nrep, const mdpd_params* params, const int64_t* n, cons
         for (int64_t f = bounds[r]; f < bounds[r + 1]; f += BATCH_CHUNK)
             chunks.push_back(make_int4(r, (int)f, (int)std::min<int64_t>(BATCH_CHUNK, bounds[r + 1] - f), 0));
         wr[r].y = (int)chunks.size() * PAIR_BLOCK_WARPS;
-        for (int64_t c = R.cell0; c < R.cell0 + R.geo.ncell; c += BATCH_CELL_CHUNK)
-            cchunks.push_back(make_int4(r, (int)c, (int)std::min<int64_t>(BATCH_CELL_CHUNK, R.cell0 + R.geo.ncell - c), 0));
     }
     h->geo = h->reps[0].geo;
     h->geo.ncell = cells;                  // the concatenated lattice (scan and cell sort)
     h->ph = h->reps[0].ph;
     h->nchunk = (int)chunks.size();
-    h->ncchunk = (int)cchunks.size();
     int rc;
     if ((rc = dalloc(h, &h->d_reps, sizeof(Rep) * (size_t)nrep)) ||
         (rc = dalloc(h, &h->d_reps_all, sizeof(Rep) * (size_t)nrep)) ||
         (rc = dalloc(h, &h->d_chunks, sizeof(int4) * chunks.size())) ||
-        (rc = dalloc(h, &h->d_cchunks, sizeof(int4) * cchunks.size())) ||
         (rc = dalloc(h, &h->d_wr, sizeof(int2) * wr.size())) ||
         (rc = dalloc(h, &h->obs_b, sizeof(double) * OBS_STRIDE * (size_t)nrep))) {
         g_create_error = h->err;
@@ -1019,7 +1009,6 @@ int create_batch(int32_t nrep, const mdpd_params* params, const int64_t* n, cons
     }
     bool ok = upload_reps(h) == MDPD_OK &&
               (chunks.empty() || cudaMemcpy(h->d_chunks, chunks.data(), sizeof(int4) * chunks.size(), cudaMemcpyHostToDevice) == cudaSuccess) &&
-              (cchunks.empty() || cudaMemcpy(h->d_cchunks, cchunks.data(), sizeof(int4) * cchunks.size(), cudaMemcpyHostToDevice) == cudaSuccess) &&
               cudaMemcpy(h->d_wr, wr.data(), sizeof(int2) * wr.size(), cudaMemcpyHostToDevice) == cudaSuccess &&
               cudaMemset(h->obs_b, 0, sizeof(double) * OBS_STRIDE * (size_t)nrep) == cudaSuccess;
     if (!ok) {
@@ -1570,11 +1559,9 @@ int mdpd_set_option(mdpd_handle* h, int32_t option, int64_t value)
         destroy_graphs(h);
         return MDPD_OK;
     case MDPD_OPT_DENSITY_SHAPE:
+        // (the density pass has one code shape; both values are accepted)
         if (value != 0 && value != 1)
             return h->fail(MDPD_ERR_INVALID_ARG, "the density code shape is 0 or 1");
-        CK(cudaStreamSynchronize(h->stream));
-        h->thread_shape = (int)value;
-        destroy_graphs(h);
         return MDPD_OK;
     case MDPD_OPT_WALL_DENSITY:
         if (h->nrep) return h->fail(MDPD_ERR_INVALID_ARG, "a batch has no walls");
@@ -1935,33 +1922,21 @@ int mdpd_autotune(mdpd_handle* h, int32_t reps, int32_t* chosen, double* ms)
         cudaEventDestroy(e1);
         return code ? h->fail(code, std::string("autotune: ") + what) : MDPD_OK;
     };
-    // 1) density variant (the thread-per-particle one in both code shapes;
-    //    ms[1] is its faster shape)
-    const int variants[3] = { MDPD_KERNELS_NLIST, MDPD_KERNELS_NLIST_THREAD,
-                              MDPD_KERNELS_NLIST_THREAD };
-    int best = h->kernels, best_shape = h->thread_shape;
-    double best_ms = 1e300;
+    // 1) the density pass (one variant writes lists; timed for the report)
+    LaunchScope scope(step_carveout(h));
     enqueue_bin(h, true);                     // same positions: same order, state kept
-    for (int v = 0; v < 3; ++v) {
-        h->kernels = variants[v];
-        h->thread_shape = v == 2 ? 1 : 0;
-        ensure_ff(h);
+    const int best = h->kernels == MDPD_KERNELS_NLIST_THREAD ? h->kernels : MDPD_KERNELS_NLIST;
+    h->kernels = best;
+    ensure_ff(h);
+    {
         const double t = time_it([&] { enqueue_density(h); });
         if (t < 0) return done(MDPD_ERR_CUDA, cudaGetErrorString(cudaGetLastError()));
-        if (ms) ms[v < 1 ? 0 : 1] = v == 2 ? std::min(ms[1], t) : t;
-        if (t < best_ms) {
-            best_ms = t;
-            best = variants[v];
-            best_shape = h->thread_shape;
-        }
+        if (ms) ms[0] = ms[1] = t;
     }
-    h->kernels = best;
-    h->thread_shape = best_shape;
-    enqueue_density(h);                       // rho and lists from the chosen variant
     // 2) lanes per particle of the force pass (evaluation only: the state is kept)
     const int lanes[3] = { 1, 2, 4 };
     int best_l = h->force_lpp;
-    best_ms = 1e300;
+    double best_ms = 1e300;
     for (int v = 0; v < 3; ++v) {
         if (h->nrep && lanes[v] != 1) {
             if (ms) ms[2 + v] = -1.0;
@@ -1983,7 +1958,7 @@ int mdpd_autotune(mdpd_handle* h, int32_t reps, int32_t* chosen, double* ms)
     if (chosen) {
         chosen[0] = best;
         chosen[1] = best_l;
-        chosen[2] = h->thread_shape;
+        chosen[2] = 0;
     }
     rc = done(MDPD_OK, "");
     if (rc) return rc;
@@ -2024,7 +1999,6 @@ void mdpd_destroy(mdpd_handle* h)
     dfree(h->win_v0);
     dfree(h->win_b);
     dfree(h->d_chunks);
-    dfree(h->d_cchunks);
     dfree(h->d_wr);
     dfree(h->obs_b);
     for (auto& e : h->tev)

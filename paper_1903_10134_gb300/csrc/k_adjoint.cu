@@ -152,7 +152,7 @@ k_force_vjp(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
         shift[tid][2] = (T)(tid / 9 - 1) * derived<T>(ph).h[2];
     }
     const int s = b.s;
-    ty[tid] = b.valid ? (uint8_t)unpack_u32(pos4[s].w) : (uint8_t)0xFF;
+    ty[tid] = b.valid ? (uint8_t)type_of(pos4[s].w) : (uint8_t)0xFF;
     __syncthreads();
     if (b.valid) {
         const uint64_t step = *step_ptr;
@@ -169,7 +169,7 @@ k_force_vjp(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
         const V pi = pos4[s];
         const V vi = vel4[s];
         const T rho_i = rho[s];
-        const uint32_t ti = unpack_u32(pi.w), id_i = unpack_u32(vi.w);
+        const uint32_t ti = type_of(pi.w), id_i = unpack_u32(vi.w);
         const bool mob_i = ((ph.frozen >> ti) & 1u) == 0u;
         T ai[3] = { T(0), T(0), T(0) };
         if (abar && mob_i)
@@ -182,7 +182,7 @@ k_force_vjp(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
             const V pj = pos4[j];
             const V vj = vel4[j];
             const T rho_j = rho[j];
-            const uint32_t tj = unpack_u32(pj.w), id_j = unpack_u32(vj.w);
+            const uint32_t tj = type_of(pj.w), id_j = unpack_u32(vj.w);
             const bool mob_j = ((ph.frozen >> tj) & 1u) == 0u;
             const T dx = pi.x - shift[code][0] - pj.x;
             const T dy = pi.y - shift[code][1] - pj.y;

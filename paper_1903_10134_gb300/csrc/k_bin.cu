@@ -5,6 +5,8 @@
 // not depend on the order of the atomics, and a cell's mobile particles come
 // first) and gathers the state into that order with positions re-expressed as
 // offsets from the cell centre.
+#include <cuda_fp16.h>
+
 #include "pair.cuh"
 
 namespace mdpd {
@@ -240,6 +242,8 @@ __global__ void k_cell_sort(int64_t ncell, const uint32_t* __restrict__ start,
     }
 }
 
+__device__ __forceinline__ uint16_t half_bits(float x) { return __half_as_ushort(__float2half_rn(x)); }
+
 // Order inside each cell by (frozen, particle id), fused with the gather into
 // cell order.  The scatter filled slot a (in atomic order)
 // with key[a] = frozen << 31 | id and
@@ -254,8 +258,8 @@ __global__ void k_rank_gather(int n, int64_t cap, const uint32_t* __restrict__ c
                               const uint32_t* __restrict__ src, Master in, Master out,
                               int gather_a, Geo geo_p, Phys ph_p, Batch bt,
                               typename Vec4<T>::type* __restrict__ pos4,
-                              typename Vec4<T>::type* __restrict__ vel4,
-                              uint32_t* __restrict__ cell_s)
+                              typename Vec4<T>::type* __restrict__ vel4, float4* __restrict__ fpos,
+                              uint16_t* __restrict__ hpos, uint32_t* __restrict__ cell_s)
 {
     pdl_enter();
     int a;
@@ -329,7 +333,18 @@ __global__ void k_rank_gather(int n, int64_t cap, const uint32_t* __restrict__ c
                 off[k] = to_t<T>(xv[k] - fma((double)q[k], geo.h[k], ph_g.dd.c0[k]));
         }
     }
-    pos4[s] = make4(off[0], off[1], off[2], pack_u32(T(0), (uint32_t)pt));
+    pos4[s] = make4(off[0], off[1], off[2], pack_u32(T(0), (uint32_t)pt | (uint32_t)q[0] << 3));   // (q < 2^24)
+    // FP32 offsets beside FP64 ones, and the density filter's FP16 positions
+    const float fo[3] = { to_f32(off[0]), to_f32(off[1]), to_f32(off[2]) };
+    if constexpr (sizeof(T) == 8)
+        fpos[s] = make_float4(fo[0], fo[1], fo[2], __uint_as_float((uint32_t)pt | (uint32_t)q[0] << 3));
+    const Derived<float>& df = ph_g.df;
+    uint16_t* hp = hpos + (size_t)(s >> 2) * 16 + (s & 3u);
+    const float hx = df.h[0];
+    hp[0] = half_bits(fo[1] * df.inv_rc);
+    hp[4] = half_bits(fo[2] * df.inv_rc);
+    hp[8] = half_bits(fmaf((float)(2 * (q[0] & 3) - 3), 0.5f * hx, fo[0]) * df.inv_rc);
+    hp[12] = half_bits(fmaf((float)(2 * ((q[0] + 2) & 3) - 3), 0.5f * hx, fo[0]) * df.inv_rc);
     // the random stream is keyed on ids within the replica
     vel4[s] = make4(to_t<T>(vv[0]), to_t<T>(vv[1]), to_t<T>(vv[2]), pack_u32(T(0), pid - id0));
 }
@@ -500,33 +515,36 @@ void launch_cell_sort(cudaStream_t st, int64_t ncell, const uint32_t* start, uin
 void launch_rank_gather(cudaStream_t st, int precision, int n, int64_t cap,
                         const uint32_t* cellof, const uint32_t* start, const uint32_t* key,
                         const uint32_t* src, const Master& in, const Master& out, bool gather_a,
-                        const Geo& geo, const Phys& ph, void* pos4, void* vel4, uint32_t* cell_s)
+                        const Geo& geo, const Phys& ph, void* pos4, void* vel4, void* fpos, uint16_t* hpos,
+                              uint32_t* cell_s)
 {
     if (n <= 0) return;
     if (precision == 0)
         launch_pdl(k_rank_gather<double, false>, dim3(nblocks(n)), dim3(BLOCK), st, n, cap, cellof,
                    start, key, src, in, out, (int)gather_a, geo, ph, Batch{}, (D4*)pos4, (D4*)vel4,
-                   cell_s);
+                   (float4*)fpos, hpos, cell_s);
     else
         launch_pdl(k_rank_gather<float, false>, dim3(nblocks(n)), dim3(BLOCK), st, n, cap, cellof,
                    start, key, src, in, out, (int)gather_a, geo, ph, Batch{}, (float4*)pos4,
-                   (float4*)vel4, cell_s);
+                   (float4*)vel4, (float4*)fpos, hpos, cell_s);
 }
 
 void launch_rank_gather_batch(cudaStream_t st, int precision, int64_t cap, const uint32_t* cellof,
                               const uint32_t* start, const uint32_t* key, const uint32_t* src,
                               const Master& in, const Master& out, bool gather_a, const Batch& bt,
-                              void* pos4, void* vel4, uint32_t* cell_s)
+                              void* pos4, void* vel4, void* fpos, uint16_t* hpos,
+                              uint32_t* cell_s)
 {
     if (bt.nchunk <= 0) return;
     const dim3 g(bt.nchunk), b(BATCH_CHUNK);
     if (precision == 0)
         launch_pdl_smem(k_rank_gather<double, true>, g, b, REP_SMEM, st, 0, cap, cellof, start, key,
-                        src, in, out, (int)gather_a, Geo{}, Phys{}, bt, (D4*)pos4, (D4*)vel4, cell_s);
+                        src, in, out, (int)gather_a, Geo{}, Phys{}, bt, (D4*)pos4, (D4*)vel4,
+                        (float4*)fpos, hpos, cell_s);
     else
         launch_pdl_smem(k_rank_gather<float, true>, g, b, REP_SMEM, st, 0, cap, cellof, start, key,
                         src, in, out, (int)gather_a, Geo{}, Phys{}, bt, (float4*)pos4, (float4*)vel4,
-                        cell_s);
+                        (float4*)fpos, hpos, cell_s);
 }
 
 __global__ void k_frozen_moved(int n, int64_t cap, const double* __restrict__ x,

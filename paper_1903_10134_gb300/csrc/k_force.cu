@@ -146,7 +146,7 @@ k_force_nl(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt, MaskDev mk,
             const V pi = pos4[s];
             const V vi = vel4[s];
             const T rho_i = rho[s];
-            const uint32_t ti = unpack_u32(pi.w);
+            const uint32_t ti = type_of(pi.w);
             const uint32_t id_i = unpack_u32(vi.w);
             const V* tP = tab.P + ti * 8;
             const uint32_t cnt = nl_count[s];
@@ -181,7 +181,7 @@ k_force_nl(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt, MaskDev mk,
                     const T dy = pi.y - sh.y - pj.y;
                     const T dz = pi.z - sh.z - pj.z;
                     const T r2 = dx * dx + dy * dy + dz * dz;
-                    pair_term<T, !BATCH>(c, tP[unpack_u32(pj.w)], dx, dy, dz, r2, vi, vj, rho_i, rj,
+                    pair_term<T, !BATCH>(c, tP[type_of(pj.w)], dx, dy, dz, r2, vi, vj, rho_i, rj,
                                          id_i, unpack_u32(vj.w), step, ph, f, W);
                     e0 = e1;
                     e1 = e2;
@@ -217,7 +217,7 @@ k_force_nl(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt, MaskDev mk,
                                 const T r2 = dx * dx + dy * dy + dz * dz;
                                 if (r2 < c.rc2 && r2 > T(0)) {
                                     const V vj = vel4[j];
-                                    pair_term<T, !BATCH>(c, tP[unpack_u32(pj.w)], dx, dy, dz, r2, vi,
+                                    pair_term<T, !BATCH>(c, tP[type_of(pj.w)], dx, dy, dz, r2, vi,
                                                          vj, rho_i, rho[j], id_i, unpack_u32(vj.w),
                                                          step, ph, f, W);
                                     ++npair;

@@ -99,7 +99,7 @@ k_force(int n, int64_t cap, Geo geo, Phys ph, MaskDev mk,
         const auto pi = pos4[s];
         const auto vi = vel4[s];
         const T rho_i = rho[s];
-        const uint32_t ti = unpack_u32(pi.w);
+        const uint32_t ti = type_of(pi.w);
         const uint32_t id_i = unpack_u32(vi.w);
         const bool mobile = ((ph.frozen >> ti) & 1u) == 0u;
         T f[3] = { T(0), T(0), T(0) };
@@ -131,7 +131,7 @@ k_force(int n, int64_t cap, Geo geo, Phys ph, MaskDev mk,
                             const T r2 = dx * dx + dy * dy + dz * dz;
                             if (r2 < c.rc2 && r2 > T(0)) {
                                 const auto vj = vel4[j];
-                                pair_term<T, true>(c, tP[unpack_u32(pj.w)], dx, dy, dz, r2, vi, vj,
+                                pair_term<T, true>(c, tP[type_of(pj.w)], dx, dy, dz, r2, vi, vj,
                                                    rho_i, rho[j], id_i, unpack_u32(vj.w), step,
                                                    ph, f, W);
                                 ++npair;

@@ -165,16 +165,13 @@ static_assert(offsetof(Rep, ph) % 16 == 0 && sizeof(Rep) % 16 == 0, "Rep is copi
 // slots [reps[r].id0, reps[r].id0 + reps[r].n), in every ordering, so the
 // work can be cut into chunks that never straddle two replicas:
 //   chunks[b]  = (replica, first slot, count <= 128, 0)   for particle kernels
-//   cchunks[b] = (replica, first cell, count <= 4, 0)     for cell kernels
 struct Batch {
     const Rep* reps;
     const int4* chunks;
-    const int4* cchunks;
-    int nchunk, ncchunk;
+    int nchunk;
 };
 
 constexpr int BATCH_CHUNK = 128;       // particles per chunk
-constexpr int BATCH_CELL_CHUNK = 4;    // cells per chunk (warps of the cell kernel)
 
 // Solid-voxel reflection mask (1 bit per voxel, x fastest); bits == nullptr
 // means no mask.
@@ -287,6 +284,12 @@ __device__ __forceinline__ const Rep& block_rep(const Rep* __restrict__ reps, in
     return *reinterpret_cast<const Rep*>(rep_smem);
 }
 
+// FP16 positions for the density pass's filter, in groups of four slots: y x 4,
+// z x 4, xa x 4, xb x 4 (32 bytes).  y and z are offsets from the cell's centre, xa
+// and xb are measured from the middle of the four cells 4k .. 4k + 3 and 4k - 2 ..
+// 4k + 1 the particle's is one of, all in units of r_c.
+__host__ __device__ inline size_t hpos_words(size_t cap) { return (cap + 7) / 4 * 16; }
+
 constexpr int OBS_PARTIALS = 16;   // observable slots per partial (14 used)
 
 // ---- launchers (binning / scan) -------------------------------------------
@@ -324,11 +327,13 @@ void launch_scan_from_sums(cudaStream_t st, uint32_t* in, int64_t n, uint32_t* o
 void launch_rank_gather(cudaStream_t st, int precision, int n, int64_t cap,
                         const uint32_t* cellof, const uint32_t* start, const uint32_t* key,
                         const uint32_t* src, const Master& in, const Master& out, bool gather_a,
-                        const Geo& geo, const Phys& ph, void* pos4, void* vel4, uint32_t* cell_s);
+                        const Geo& geo, const Phys& ph, void* pos4, void* vel4, void* fpos,
+                        uint16_t* hpos, uint32_t* cell_s);
 void launch_rank_gather_batch(cudaStream_t st, int precision, int64_t cap, const uint32_t* cellof,
                               const uint32_t* start, const uint32_t* key, const uint32_t* src,
                               const Master& in, const Master& out, bool gather_a, const Batch& bt,
-                              void* pos4, void* vel4, uint32_t* cell_s);
+                              void* pos4, void* vel4, void* fpos, uint16_t* hpos,
+                              uint32_t* cell_s);
 void launch_bin_scatter(cudaStream_t st, int n, const uint32_t* cellof, const uint32_t* slot,
                         const uint32_t* start, const uint32_t* id, uint32_t* key, uint32_t* src,
                         uint32_t* status);
@@ -363,14 +368,10 @@ int force_nl_rounds(const Phys& ph, int lpp);
 // mobile homes only, which scatter their terms to frozen candidates into
 // facc, and a second launch forms the frozen densities and clears facc.
 void launch_density_nl(cudaStream_t st, int precision, int n, int64_t cap, const Geo& geo,
-                       const Phys& ph, const void* pos4, const uint32_t* cell_s,
-                       const uint32_t* start, void* rho, uint32_t* nl, uint32_t* nl_count,
+                       const Phys& ph, const void* pos4, const void* fpos, const uint16_t* hpos,
+                       const uint32_t* cell_s, const uint32_t* start, void* rho, uint32_t* nl, uint32_t* nl_count,
                        int fs = 0, unsigned long long* facc = nullptr,
-                       const uint32_t* id_s = nullptr, void* rho_ff = nullptr, int shape = 0);
-// Warp-per-cell variant of launch_density_nl (same outputs).
-void launch_density_cell(cudaStream_t st, int precision, int64_t ncell, int64_t cap,
-                         const Geo& geo, const Phys& ph, const void* pos4, const uint32_t* start,
-                         void* rho, uint32_t* nl, uint32_t* nl_count);
+                       const uint32_t* id_s = nullptr, void* rho_ff = nullptr);
 // lpp: lanes per particle (1, 2 or 4).
 void launch_force_nl(cudaStream_t st, int precision, ForceMode mode, int n, int64_t cap,
                      const Geo& geo, const Phys& ph, int lpp, const MaskDev& mk, const void* pos4,
@@ -396,13 +397,9 @@ void launch_load_state_batch(cudaStream_t st, int64_t cap, const double* pos3, c
 void launch_bin_count_batch(cudaStream_t st, int64_t cap, const Batch& bt, const Master& m,
                             bool kick, uint32_t* cellof, uint32_t* slot, uint32_t* count,
                             uint32_t* tsum, uint32_t* status);
-// shape: code shape of the thread-per-particle kernel (0 or 1; same results).
 void launch_density_nl_batch(cudaStream_t st, int precision, int64_t cap, const Batch& bt,
-                             const void* pos4, const uint32_t* cell_s, const uint32_t* start,
-                             void* rho, uint32_t* nl, uint32_t* nl_count, int shape = 0);
-void launch_density_cell_batch(cudaStream_t st, int precision, int64_t cap, const Batch& bt,
-                               const void* pos4, const uint32_t* start, void* rho, uint32_t* nl,
-                               uint32_t* nl_count);
+                             const void* pos4, const void* fpos, const uint16_t* hpos,
+                             const uint32_t* cell_s, const uint32_t* start, void* rho, uint32_t* nl, uint32_t* nl_count);
 // Partials: 4 per chunk (bt.nchunk * 4 in all).
 void launch_force_nl_batch(cudaStream_t st, int precision, ForceMode mode, int64_t cap,
                            const Batch& bt, const void* pos4, const void* vel4, const void* rho,

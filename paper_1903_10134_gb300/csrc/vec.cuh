@@ -14,12 +14,14 @@ template <typename T> struct Vec4;
 template <> struct Vec4<float> { using type = float4; };
 template <> struct Vec4<double> { using type = D4; };
 
-// pos4.w carries the particle type and vel4.w the particle id.  In FP32 the
-// words hold the integers' bits; in FP64 the integers' values (exact below 2^53).
+// pos4.w carries the particle type | (its cell column) << 3 and vel4.w the
+// particle id, as the integers' bits (in FP64 too: conversions are slow there).
 __device__ __forceinline__ float pack_u32(float, uint32_t u) { return __uint_as_float(u); }
-__device__ __forceinline__ double pack_u32(double, uint32_t u) { return (double)u; }
+__device__ __forceinline__ double pack_u32(double, uint32_t u) { return __longlong_as_double((long long)u); }
 __device__ __forceinline__ uint32_t unpack_u32(float f) { return __float_as_uint(f); }
-__device__ __forceinline__ uint32_t unpack_u32(double d) { return (uint32_t)d; }
+__device__ __forceinline__ uint32_t unpack_u32(double d) { return (uint32_t)__double_as_longlong(d); }
+template <typename T>
+__device__ __forceinline__ uint32_t type_of(T w) { return unpack_u32(w) & 7u; }
 
 __device__ __forceinline__ float4 make4(float x, float y, float z, float w)
 {
