@@ -542,7 +542,7 @@ void ensure_ff(mdpd_handle* h)
 
 // Partner lists indexed by compacted mobile position (ph.list_compact): the
 // frozen-split density pass and the force pass at one lane per particle use
-// the same blocks of FORCE_ROUNDS * PAIR_BLOCK slots.
+// the same blocks of slots (frozen_rounds).
 bool list_compact(const mdpd_handle* h) { return use_split(h) && h->force_lpp == 1; }
 
 // all: partner lists for every particle, frozen ones too (the adjoint's;
@@ -594,7 +594,7 @@ void enqueue_reduce(mdpd_handle* h, int advance, cudaStream_t st = nullptr)
     }
     const bool scan = h->kernels == MDPD_KERNELS_SCAN;
     const int lpp = scan ? 1 : h->force_lpp;
-    const int rounds = scan ? 1 : force_nl_rounds(h->ph, lpp);
+    const int rounds = scan ? 1 : force_nl_rounds(h->ph, lpp, h->n);
     launch_reduce_obs(st, h->precision, h->partials, obs_num_partials((int)h->n, lpp, rounds),
                       h->red_l1,
                       h->red_ticket, h->obs, h->obs + MDPD_NUM_OBS, h->obs + 2 * MDPD_NUM_OBS,

@@ -138,8 +138,15 @@ k_frozen_part(int n, int64_t cap, Geo geo, Phys ph, const typename Vec4<T>::type
 // Runs and masks wait in shared memory, in one array: the masks of the runs done
 // (empty ones skipped) take the places of those runs.  A home with more masks than
 // that (runs longer than 32 candidates) works them off and goes on.
-constexpr int DN_RUNS = 18;
-constexpr int DN_NEAR = 32;        // FP64: listed candidates near r_d kept per home
+//
+// LPH lanes share a home in small systems (density_lanes), where one lane's chain of
+// 5,000 instructions is the pass's time: the lanes take the rows 0 - 3, 4 (its own, with
+// ten of the 25 hits), 5 - 6 and 7 - 8, and their hits and density terms wait in
+// shared memory.  The list
+// is then the lanes' hits one after another and one lane adds the terms in that
+// order, so lists and sums are those of one lane.  A home whose lanes' hits do not
+// fit is done again by one lane after the other.
+constexpr int DN_HITS = 24;        // hits and terms kept per lane (LPH > 1)
 // r^2 < FILT passes (1 + 9 * 2^-10, exact in FP16).  With u = 2^-10 an |x| < 4 is off by
 // u at most, home and candidate; |y|, |z| < 1 of a candidate by u / 4, < 3 of a home
 // by u; a difference near 1 by u / 2 more.  That is 2.5 u in x and 1.75 u in y and z,
@@ -147,16 +154,28 @@ constexpr int DN_NEAR = 32;        // FP64: listed candidates near r_d kept per 
 // u / 2: below 8 u.
 constexpr float FILT = 1.0f + 9.0f / 1024.0f;
 
-template <typename T>
+template <typename T, int LPH>
 struct DensitySmem {
+    static constexpr int RUNS = LPH == 1 ? 18 : 8;     // two for each of a lane's rows
+    // FP64: candidates near r_d kept before they are evaluated
+    static constexpr int NEAR = sizeof(T) == 4 ? 1 : 32;
     // run: length, first slot | row << 27 | across a face in x << 31
     // mask: candidates from the top bit, first slot | row << 27 | across << 31
-    uint32_t a[DN_RUNS][PAIR_BLOCK];
-    uint32_t b[DN_RUNS][PAIR_BLOCK];
+    uint32_t a[RUNS][PAIR_BLOCK];
+    uint32_t b[RUNS][PAIR_BLOCK];
     typename Vec4<T>::type shift[27];          // image shift of a neighbour-cell code
     float4 fshift[sizeof(T) == 8 ? 27 : 1];    // the same in FP32
-    uint32_t near[sizeof(T) == 8 ? DN_NEAR : 1][PAIR_BLOCK];
+    uint32_t near[NEAR][PAIR_BLOCK];
+    uint32_t hit[LPH == 1 ? 1 : DN_HITS][PAIR_BLOCK];
+    T term[LPH == 1 ? 1 : DN_HITS][PAIR_BLOCK];
 };
+
+// Density terms and sums with each operation rounded, so that the two ways of
+// adding them (LPH) agree.
+__device__ __forceinline__ float rho_term(float cw, float w) { return __fmul_rn(__fmul_rn(cw, w), w); }
+__device__ __forceinline__ double rho_term(double cw, double w) { return __dmul_rn(__dmul_rn(cw, w), w); }
+__device__ __forceinline__ float rho_add(float a, float t) { return __fadd_rn(a, t); }
+__device__ __forceinline__ double rho_add(double a, double t) { return __dadd_rn(a, t); }
 
 // k as a float for k < 2^23 (the conversion instruction runs at an eighth of the rate)
 __device__ __forceinline__ float small_float(uint32_t k)
@@ -176,8 +195,8 @@ __device__ __forceinline__ uint32_t push_signs(uint32_t m, __half2 t01, __half2 
 }
 __device__ __forceinline__ __half2 as_half2(uint32_t u) { return *reinterpret_cast<__half2*>(&u); }
 
-template <typename T>
-__device__ __forceinline__ void fill_shift(DensitySmem<T>& sm, const Phys& ph)
+template <typename T, int LPH>
+__device__ __forceinline__ void fill_shift(DensitySmem<T, LPH>& sm, const Phys& ph)
 {
     const int c = threadIdx.x;
     if (c >= 27) return;
@@ -190,39 +209,47 @@ __device__ __forceinline__ void fill_shift(DensitySmem<T>& sm, const Phys& ph)
 }
 
 // The density and partner list of the home in slot s; column lcol of the list.
-template <typename T, bool WANT_PHI, int FS>
+// With LPH > 1 the LPH lanes of a group call it together.
+template <typename T, bool WANT_PHI, int FS, int LPH>
 __device__ __forceinline__ void density_home(
-    DensitySmem<T>& sm, int s, int64_t cap, const Geo& geo, const Phys& ph, int64_t cell0,
+    DensitySmem<T, LPH>& sm, int s, int64_t cap, const Geo& geo, const Phys& ph, int64_t cell0,
     const typename Vec4<T>::type* __restrict__ pos4, const float4* __restrict__ fpos,
-    const uint4* __restrict__ hpos, const uint32_t* __restrict__ cell_s, const uint32_t* __restrict__ start,
-    T* __restrict__ rho_out, uint32_t* __restrict__ nl, uint32_t* __restrict__ nl_count,
-    unsigned long long* __restrict__ facc, int64_t lcol)
+    const uint4* __restrict__ hpos, const uint32_t* __restrict__ cell_s,
+    const uint32_t* __restrict__ start, T* __restrict__ rho_out, uint32_t* __restrict__ nl,
+    uint32_t* __restrict__ nl_count, unsigned long long* __restrict__ facc, int64_t lcol)
 {
+    static_assert(LPH == 1 || LPH == 4, "lanes per home");
     const Derived<T>& dc = derived<T>(ph);
     const Derived<float>& df = ph.df;
     const int tid = threadIdx.x;
+    const int sub = LPH == 1 ? 0 : tid % LPH;
+    const unsigned group = LPH == 1 ? 0u : ((1u << LPH) - 1u) << ((tid & 31) & ~(LPH - 1));
     const auto pi = pos4[s];
     int q0, q1, q2;
     cell_coords(cell_s[s], geo, q0, q1, q2);
 
     // the runs: rows (oy, oz) in order, the part across the lower face in x first,
     // the part across the upper one last
+    const bool lo_x = geo.periodic[0] && q0 == 0, hi_x = geo.periodic[0] && q0 == geo.nc[0] - 1;
+    const int xb0 = max(q0 - 1, 0), xe0 = min(q0 + 1, geo.nc[0] - 1) + 1;
+    constexpr int ROWS = LPH == 1 ? 9 : 4;
+    const int row0 = LPH == 1 ? 0 : (0x97540 >> 4 * sub) & 15, row1 = LPH == 1 ? 9 : (0x9754 >> 4 * sub) & 15;
     int nrun = 0;
-    {
-        const bool lo_x = geo.periodic[0] && q0 == 0, hi_x = geo.periodic[0] && q0 == geo.nc[0] - 1;
-        const int xb = max(q0 - 1, 0), xe = min(q0 + 1, geo.nc[0] - 1) + 1;
-        uint32_t b[9], e[9];
-#pragma unroll
-        for (int r = 0; r < 9; ++r) {
+    auto build_runs = [&]() {
+        uint32_t b[ROWS], e[ROWS];
+        auto row_start = [&](int r) -> const uint32_t* {
             const int z = neighbour_index(q2, r / 3 - 1, geo.nc[2], geo.periodic[2]);
             const int y = neighbour_index(q1, r % 3 - 1, geo.nc[1], geo.periodic[1]);
-            const uint32_t* st = start + cell0 + geo.nc[0] * (y + geo.nc[1] * z);
-            b[r] = e[r] = 0u;
-            if (z >= 0 && y >= 0) {
-                b[r] = st[xb];
-                e[r] = st[xe];
-            }
+            return r < row1 && z >= 0 && y >= 0 ? start + cell0 + geo.nc[0] * (y + geo.nc[1] * z)
+                                                : nullptr;
+        };
+#pragma unroll
+        for (int k = 0; k < ROWS; ++k) {
+            const uint32_t* st = row_start(row0 + k);
+            b[k] = st ? st[xb0] : 0u;
+            e[k] = st ? st[xe0] : 0u;
         }
+        nrun = 0;
         auto put = [&](uint32_t first, uint32_t end, uint32_t code) {
             if (first < end && MDPD_DBG_OK(end <= (uint32_t)cap, ph.dbg_status)) {
                 sm.a[nrun][tid] = end - first;
@@ -231,21 +258,20 @@ __device__ __forceinline__ void density_home(
             }
         };
 #pragma unroll
-        for (int r = 0; r < 9; ++r) {
+        for (int k = 0; k < ROWS; ++k) {
+            const uint32_t r = (uint32_t)(row0 + k);
             if (lo_x || hi_x) {
-                const int z = neighbour_index(q2, r / 3 - 1, geo.nc[2], geo.periodic[2]);
-                const int y = neighbour_index(q1, r % 3 - 1, geo.nc[1], geo.periodic[1]);
-                if (z < 0 || y < 0) continue;
-                const uint32_t* st = start + cell0 + geo.nc[0] * (y + geo.nc[1] * z);
+                const uint32_t* st = row_start((int)r);
+                if (!st) continue;
                 const int x = lo_x ? geo.nc[0] - 1 : 0;
-                if (hi_x) put(b[r], e[r], r);
+                if (hi_x) put(b[k], e[k], r);
                 put(st[x], st[x + 1], r | 16u);
-                if (lo_x) put(b[r], e[r], r);
+                if (lo_x) put(b[k], e[k], r);
             } else {
-                put(b[r], e[r], r);
+                put(b[k], e[k], r);
             }
         }
-    }
+    };
     const bool mob_true = ((ph.frozen >> type_of(pi.w)) & 1u) == 0u;
     const bool mobile = ph.list_all || mob_true;
     // wall density of a mobile particle (WANT_PHI): sum over frozen partners
@@ -272,6 +298,13 @@ __device__ __forceinline__ void density_home(
     __half2 hx = hx0, hy = hx0, hz = hx0;
     bool xb = win_b;
 
+    // pass 0: every lane its rows (LPH > 1: hits and terms kept); passes 1 .. LPH, if
+    // a lane's did not fit: the lanes in turn, straight to the list and the sum
+    uint32_t nhit = 0, nterm = 0;
+    for (int pass = 0; pass <= (LPH == 1 ? 0 : LPH); ++pass) {
+    const bool keep = LPH > 1 && pass == 0;
+    if (LPH == 1 || pass == 0 || sub == pass - 1) {
+    build_runs();
     int run = 0;
     uint32_t len = 0, rb = 0;
     while (run < nrun || len) {
@@ -342,9 +375,25 @@ __device__ __forceinline__ void density_home(
             return 3 * (int)((jr >> 27) & 15u) + ox + 1;
         };
         auto append = [&](uint32_t j, int code) {
-            if (cnt < (uint32_t)NL_MAX) *lp = j << 5 | (uint32_t)code;
+            const uint32_t entry = j << 5 | (uint32_t)code;   // (bits above the slot shift out)
+            if (LPH > 1 && keep) {
+                if (nhit < (uint32_t)DN_HITS) sm.hit[nhit][tid] = entry;
+                ++nhit;
+                return;
+            }
+            if (cnt < (uint32_t)NL_MAX) *lp = entry;
             lp += cap;
             ++cnt;
+        };
+        auto add = [&](T term) {
+            if (LPH > 1 && keep) {
+                if (term > T(0)) {
+                    if (nterm < (uint32_t)DN_HITS) sm.term[nterm][tid] = term;
+                    ++nterm;
+                }
+                return;
+            }
+            acc = rho_add(acc, term);
         };
         next();
         if constexpr (sizeof(T) == 4) {
@@ -365,14 +414,14 @@ __device__ __forceinline__ void density_home(
                 const float r2 = dx * dx + dy * dy + dz * dz;
                 if (r2 < dc.rc2) {
                     const float wr = max(1.0f - sqrt_fast(r2) * dc.inv_rd, 0.0f);
-                    const float term = dc.cw_rho * wr * wr;      // r = 0 gives w(0)
-                    acc += term;
+                    const float term = rho_term(dc.cw_rho, wr);  // r = 0 gives w(0)
+                    add(term);
                     const bool fz = (FS == 1 || WANT_PHI) && ((ph.frozen >> (bits & 7u)) & 1u);
-                    if (FS == 1 && fz && term > 0.0f)
+                    if (FS == 1 && fz && term > 0.0f && pass == 0)
                         atomicAdd(facc + (jr & 0x07ffffffu), to_fixed(term * dc.fix_scale));
                     if (mobile && r2 > 0.0f) {      // not the home, not coincident
-                        append(jr, code);           // (the bits above the slot shift out)
-                        if (want_phi && fz) {
+                        append(jr, code);
+                        if (want_phi && fz && pass == 0) {
                             const float wq = 1.0f - sqrt_t(r2) * dc.inv_rc;
                             phi += dc.cw_phi * wq * wq;
                         }
@@ -398,9 +447,9 @@ __device__ __forceinline__ void density_home(
                 const T r2 = r2_of(j, (int)(entry & 31u));
                 if (r2 < dc.rc2) {
                     const T wr = max(T(1) - sqrt_fast(r2) * dc.inv_rd, T(0));
-                    const T term = dc.cw_rho * wr * wr;          // r = 0 gives w(0)
-                    acc += term;
-                    const bool fz = (FS == 1 || WANT_PHI) &&
+                    const T term = rho_term(dc.cw_rho, wr);      // r = 0 gives w(0)
+                    add(term);
+                    const bool fz = (FS == 1 || WANT_PHI) && pass == 0 &&
                                     ((ph.frozen >> type_of(pos4[j].w)) & 1u);
                     if (FS == 1 && fz && term > T(0))
                         atomicAdd(facc + j, to_fixed(term * dc.fix_scale));
@@ -409,6 +458,10 @@ __device__ __forceinline__ void density_home(
                         phi += dc.cw_phi * wq * wq;
                     }
                 }
+            };
+            auto evaluate_near = [&]() {
+                for (int k = 0; k < nnear; ++k) evaluate(sm.near[k][tid]);
+                nnear = 0;
             };
             float4 p1 = fpos[j1 & 0x07ffffffu];
             for (;;) {
@@ -433,15 +486,48 @@ __device__ __forceinline__ void density_home(
                 }
                 if (mobile && in) append(jr, code);
                 if (!(r2 >= near2) || (want_phi && ((ph.frozen >> (bits & 7u)) & 1u))) {
-                    if (nnear < DN_NEAR) sm.near[nnear++][tid] = entry;
-                    else evaluate(entry);
+                    sm.near[nnear++][tid] = entry;
+                    if (nnear == DensitySmem<T, LPH>::NEAR) evaluate_near();
                 }
                 if (!more) break;
             }
-            for (int k = 0; k < nnear; ++k) evaluate(sm.near[k][tid]);
+            evaluate_near();
         }
     }
-    if (!ph.rho_self) acc -= dc.cw_rho;
+    }
+    if constexpr (LPH > 1) {
+        __syncwarp(group);
+        if (pass == 0) {
+            const bool fits = nhit <= (uint32_t)DN_HITS && nterm <= (uint32_t)DN_HITS;
+            // wall density: the lanes' sums in a fixed order
+            if (WANT_PHI)
+#pragma unroll
+                for (int o = 1; o < LPH; o <<= 1) phi += __shfl_xor_sync(group, phi, o);
+            if (__all_sync(group, fits)) {
+                uint32_t before = 0;
+#pragma unroll
+                for (int t = 0; t < LPH; ++t) {
+                    const uint32_t ht = __shfl_sync(group, nhit, t, LPH);
+                    const uint32_t nt = __shfl_sync(group, nterm, t, LPH);
+                    before += t < sub ? ht : 0u;
+                    cnt += ht;
+                    if (sub == 0)
+                        for (uint32_t k = 0; k < nt; ++k) acc = rho_add(acc, sm.term[k][tid + t]);
+                }
+                for (uint32_t k = 0; k < nhit; ++k)
+                    if (before + k < (uint32_t)NL_MAX) lp[(int64_t)(before + k) * cap] = sm.hit[k][tid];
+                __syncwarp(group);             // the terms are read before the next home's
+                break;
+            }
+        } else {
+            acc = __shfl_sync(group, acc, pass - 1, LPH);
+            cnt = __shfl_sync(group, cnt, pass - 1, LPH);
+            lp = nl + lcol + (int64_t)cnt * cap;
+        }
+    }
+    }
+    if (sub != 0) return;
+    if (!ph.rho_self) acc = rho_add(acc, -dc.cw_rho);
     rho_out[s] = acc;
     nl_count[s] = cnt;
     if (WANT_PHI) ((T*)ph.phi_out)[s] = phi;
@@ -455,36 +541,33 @@ __device__ __forceinline__ void density_home(
 // own) to facc[j] as a fixed-point integer (Derived::fix_scale), by atomic
 // addition, so the sum does not depend on the order; k_frozen_rho then forms
 // rho_j = rho_ff + facc * fix_inv and clears facc.  Each FS = 1 block gathers
-// the mobile homes of FS_ROUNDS * PAIR_BLOCK slots and runs them in rounds of
-// PAIR_BLOCK, so no warp is spent on frozen homes (on a porous rock about 45 %
-// of the slots are mobile, and a block of one PAIR_BLOCK would keep most of its
-// warps idle while holding its resident-block slot).  FS = 0: every particle is
+// the mobile homes of R * PAIR_BLOCK slots (R = frozen_rounds) and runs them in
+// rounds, so no warp is spent on frozen homes.  FS = 0: every particle is
 // a home, and partner lists are written for mobile ones (all under list_all).
-constexpr int FS_ROUNDS = FORCE_ROUNDS;      // the same blocks as the force pass's rounds
-
-template <typename T, bool BATCH, bool WANT_PHI, int FS>
-__global__ void __launch_bounds__(PAIR_BLOCK, sizeof(T) == 4 ? 8 : 5)
+template <typename T, bool BATCH, bool WANT_PHI, int FS, int LPH, int R>
+__global__ void __launch_bounds__(PAIR_BLOCK, LPH > 1 ? 4 : sizeof(T) == 4 ? 8 : 5)
 k_density_nl(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
              const typename Vec4<T>::type* __restrict__ pos4, const float4* __restrict__ fpos,
              const uint4* __restrict__ hpos, const uint32_t* __restrict__ cell_s,
-             const uint32_t* __restrict__ start, T* __restrict__ rho_out, uint32_t* __restrict__ nl, uint32_t* __restrict__ nl_count,
+             const uint32_t* __restrict__ start, T* __restrict__ rho_out,
+             uint32_t* __restrict__ nl, uint32_t* __restrict__ nl_count,
              unsigned long long* __restrict__ facc)
 {
     static_assert(FS == 0 || !BATCH, "the frozen split is for single systems");
-    __shared__ DensitySmem<T> sm;
+    __shared__ DensitySmem<T, LPH> sm;
+    constexpr int HOMES = PAIR_BLOCK / LPH;    // homes of a round
     pdl_enter();
     if constexpr (FS == 1) {
-        // the mobile homes of the block's FS_ROUNDS * PAIR_BLOCK slots, in
-        // slot order
-        __shared__ int act[FS_ROUNDS * PAIR_BLOCK];
-        __shared__ uint32_t wcnt[FS_ROUNDS][PAIR_BLOCK / 32];
+        // the mobile homes of the block's R * PAIR_BLOCK slots, in slot order
+        __shared__ int act[R * PAIR_BLOCK];
+        __shared__ uint32_t wcnt[R][PAIR_BLOCK / 32];
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
         const unsigned lt = (1u << lane) - 1u;
-        const int64_t base = (int64_t)blockIdx.x * (FS_ROUNDS * PAIR_BLOCK);
+        const int64_t base = (int64_t)blockIdx.x * (R * PAIR_BLOCK);
         fill_shift(sm, ph_p);
-        unsigned bm[FS_ROUNDS];
+        unsigned bm[R];
 #pragma unroll
-        for (int r = 0; r < FS_ROUNDS; ++r) {
+        for (int r = 0; r < R; ++r) {
             const int64_t t = base + r * PAIR_BLOCK + threadIdx.x;
             const bool mob = t < n && ((ph_p.frozen >> type_of(pos4[t].w)) & 1u) == 0u;
             bm[r] = __ballot_sync(0xffffffffu, mob);
@@ -493,7 +576,7 @@ k_density_nl(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
         __syncthreads();
         uint32_t nmob = 0;
 #pragma unroll
-        for (int r = 0; r < FS_ROUNDS; ++r) {
+        for (int r = 0; r < R; ++r) {
             uint32_t off = nmob;
 #pragma unroll
             for (int w = 0; w < PAIR_BLOCK / 32; ++w) {
@@ -508,84 +591,108 @@ k_density_nl(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
         // slot plus the home's place among its mobile homes, which the force
         // pass's rounds blocks form the same way (consecutive columns for a
         // warp's homes: coalesced list stores and loads)
-        for (uint32_t q = threadIdx.x; q < nmob; q += PAIR_BLOCK)
-            density_home<T, WANT_PHI, FS>(sm, act[q], cap, geo_p, ph_p, 0, pos4, fpos, hpos, cell_s,
-                                          start, rho_out, nl, nl_count, facc,
-                                          ph_p.list_compact ? base + q : (int64_t)act[q]);
+        for (uint32_t q = threadIdx.x / LPH; q < nmob; q += HOMES)
+            density_home<T, WANT_PHI, FS, LPH>(sm, act[q], cap, geo_p, ph_p, 0, pos4, fpos, hpos,
+                                               cell_s, start, rho_out, nl, nl_count, facc,
+                                               ph_p.list_compact ? base + q : (int64_t)act[q]);
         return;
     }
-    int s;
-    bool valid;
+    // a single system: one round of homes per block; a batch: a chunk's slots in rounds
+    int first, count;
     int64_t cell0 = 0;
     const Rep* rp = nullptr;
     if constexpr (BATCH) {
-        const int4 ch = bt.chunks[blockIdx.x];
+        const int4 ch = bt.chunks[blockIdx.x / LPH];
         rp = &block_rep<REP_SCALARS>(bt.reps, ch.x);
-        s = ch.y + (int)threadIdx.x;
-        valid = (int)threadIdx.x < ch.z;
+        const int part = (int)(blockIdx.x % LPH) * HOMES;
+        first = ch.y + part;
+        count = min(HOMES, ch.z - part);
         cell0 = rp->cell0;
     } else {
-        s = blockIdx.x * blockDim.x + threadIdx.x;
-        valid = s < n;
+        first = blockIdx.x * HOMES;
+        count = min(HOMES, n - first);
     }
     fill_shift(sm, BATCH ? rp->ph : ph_p);
     __syncthreads();
-    if (!valid) return;
-    density_home<T, WANT_PHI, FS>(sm, s, cap, BATCH ? rp->geo : geo_p, BATCH ? rp->ph : ph_p,
-                                  cell0, pos4, fpos, hpos, cell_s, start, rho_out, nl, nl_count, facc,
-                                  (int64_t)s);
+    const int k = (int)threadIdx.x / LPH;
+    if (k >= count) return;
+    density_home<T, WANT_PHI, FS, LPH>(sm, first + k, cap, BATCH ? rp->geo : geo_p,
+                                       BATCH ? rp->ph : ph_p, cell0, pos4, fpos, hpos, cell_s, start,
+                                       rho_out, nl, nl_count, facc, (int64_t)(first + k));
 }
 
 }  // namespace
 
-template <typename T>
+// Lanes that share a home in a pass over n slots in which every particle is a home.
+// Measured, density pass in FP32 with one lane and with four: 1,000 particles 25 and
+// 18 us, 4,000 28 and 19, 12,000 27 and 20, 20,000 27 and 29, 40,000 28 and 41.  FP64
+// (the terms of the middle row, half of them, are one lane's) 53 and 63 us at 1,000.
+static int density_lanes(int precision, int64_t n) { return precision == 1 && n <= 16000 ? 4 : 1; }
+
+template <typename T, int R>
 static void density_t(cudaStream_t st, int n, int64_t cap, const Geo& geo, const Phys& ph,
-                      const void* pos4, const void* fpos, const uint16_t* hpos, const uint32_t* cell_s,
-                      const uint32_t* start, void* rho, uint32_t* nl, uint32_t* nl_count, int fs,
-                      unsigned long long* facc, const uint32_t* id_s, void* rho_ff)
+                      const void* pos4, const void* fpos, const uint16_t* hpos,
+                      const uint32_t* cell_s, const uint32_t* start, void* rho, uint32_t* nl,
+                      uint32_t* nl_count, int fs, unsigned long long* facc, const uint32_t* id_s,
+                      void* rho_ff)
 {
     using V = typename Vec4<T>::type;
     const int nb = (n + PAIR_BLOCK - 1) / PAIR_BLOCK;
-    const int nb1 = (n + FS_ROUNDS * PAIR_BLOCK - 1) / (FS_ROUNDS * PAIR_BLOCK);
     if (fs == 2) {
         launch_pdl(k_frozen_part<T>, dim3(nb), dim3(PAIR_BLOCK), st, n, cap, geo, ph,
                    (const V*)pos4, cell_s, start, id_s, (T*)rho_ff);
         return;
     }
     const bool phi = ph.phi_out != nullptr;
-    auto k = fs == 1 ? (phi ? k_density_nl<T, false, true, 1> : k_density_nl<T, false, false, 1>)
-                     : (phi ? k_density_nl<T, false, true, 0> : k_density_nl<T, false, false, 0>);
-    launch_pdl(k, dim3(fs == 1 ? nb1 : nb), dim3(PAIR_BLOCK), st, n, cap, geo, ph, Batch{},
-               (const V*)pos4, (const float4*)fpos, (const uint4*)hpos, cell_s, start, (T*)rho, nl, nl_count, facc);
+    const int lph = fs == 1 ? 1 : density_lanes(sizeof(T) == 8 ? 0 : 1, n);
+    auto k = fs == 1 ? (phi ? k_density_nl<T, false, true, 1, 1, R> : k_density_nl<T, false, false, 1, 1, R>)
+                     : (phi ? k_density_nl<T, false, true, 0, 1, 1> : k_density_nl<T, false, false, 0, 1, 1>);
+    if constexpr (sizeof(T) == 4)
+        if (lph == 4)
+            k = phi ? k_density_nl<T, false, true, 0, 4, 1> : k_density_nl<T, false, false, 0, 4, 1>;
+    const int per = fs == 1 ? R * PAIR_BLOCK : PAIR_BLOCK / lph;      // slots of a block
+    launch_pdl(k, dim3((n + per - 1) / per), dim3(PAIR_BLOCK), st, n, cap, geo, ph, Batch{},
+               (const V*)pos4, (const float4*)fpos, (const uint4*)hpos, cell_s, start, (T*)rho, nl,
+               nl_count, facc);
     if (fs == 1)
         launch_pdl(k_frozen_rho<T>, dim3(nb), dim3(PAIR_BLOCK), st, n, ph, id_s,
                    (const T*)rho_ff, facc, (T*)rho);
 }
 
 void launch_density_nl(cudaStream_t st, int precision, int n, int64_t cap, const Geo& geo,
-                       const Phys& ph, const void* pos4, const void* fpos, const uint16_t* hpos, const uint32_t* cell_s,
-                       const uint32_t* start, void* rho, uint32_t* nl, uint32_t* nl_count,
-                       int fs, unsigned long long* facc, const uint32_t* id_s, void* rho_ff)
+                       const Phys& ph, const void* pos4, const void* fpos, const uint16_t* hpos,
+                       const uint32_t* cell_s, const uint32_t* start, void* rho, uint32_t* nl,
+                       uint32_t* nl_count, int fs, unsigned long long* facc, const uint32_t* id_s,
+                       void* rho_ff)
 {
     if (n <= 0) return;
-    auto f = precision == 0 ? density_t<double> : density_t<float>;
+    const bool rounds = frozen_rounds(n) > 1;
+    auto f = precision == 0 ? (rounds ? density_t<double, FORCE_ROUNDS> : density_t<double, 1>)
+                            : (rounds ? density_t<float, FORCE_ROUNDS> : density_t<float, 1>);
     f(st, n, cap, geo, ph, pos4, fpos, hpos, cell_s, start, rho, nl, nl_count, fs, facc, id_s, rho_ff);
 }
 
+template <typename T, int LPH>
+static void density_batch_t(cudaStream_t st, int64_t cap, const Batch& bt, const void* pos4,
+                            const void* fpos, const uint16_t* hpos, const uint32_t* cell_s,
+                            const uint32_t* start, void* rho, uint32_t* nl, uint32_t* nl_count)
+{
+    launch_pdl_smem(k_density_nl<T, true, false, 0, LPH, 1>, dim3(bt.nchunk * LPH), dim3(PAIR_BLOCK),
+                    REP_SMEM, st, 0, cap, Geo{}, Phys{}, bt, (const typename Vec4<T>::type*)pos4,
+                    (const float4*)fpos, (const uint4*)hpos, cell_s, start, (T*)rho, nl, nl_count,
+                    nullptr);
+}
+
 void launch_density_nl_batch(cudaStream_t st, int precision, int64_t cap, const Batch& bt,
-                             const void* pos4, const void* fpos, const uint16_t* hpos, const uint32_t* cell_s,
-                             const uint32_t* start, void* rho, uint32_t* nl, uint32_t* nl_count)
+                             const void* pos4, const void* fpos, const uint16_t* hpos,
+                             const uint32_t* cell_s, const uint32_t* start, void* rho, uint32_t* nl,
+                             uint32_t* nl_count)
 {
     if (bt.nchunk <= 0) return;
-    const dim3 g(bt.nchunk), b(PAIR_BLOCK);
-    if (precision == 0)
-        launch_pdl_smem(k_density_nl<double, true, false, 0>, g, b, REP_SMEM, st, 0, cap, Geo{},
-                        Phys{}, bt, (const D4*)pos4, (const float4*)fpos, (const uint4*)hpos, cell_s, start,
-                        (double*)rho, nl, nl_count, nullptr);
-    else
-        launch_pdl_smem(k_density_nl<float, true, false, 0>, g, b, REP_SMEM, st, 0, cap, Geo{},
-                        Phys{}, bt, (const float4*)pos4, (const float4*)fpos, (const uint4*)hpos, cell_s, start,
-                        (float*)rho, nl, nl_count, nullptr);
+    auto f = precision == 0 ? density_batch_t<double, 1>
+             : density_lanes(precision, (int64_t)bt.nchunk * PAIR_BLOCK) == 4 ? density_batch_t<float, 4>
+                                                                             : density_batch_t<float, 1>;
+    f(st, cap, bt, pos4, fpos, hpos, cell_s, start, rho, nl, nl_count);
 }
 
 }  // namespace mdpd

@@ -17,10 +17,11 @@ __device__ __forceinline__ int image_code(int ox, int oy, int oz)
 // consecutive in cell order) are first compacted so that the mobile ones sit
 // on the leading lanes (frozen wall particles need no force), then each of
 // those lanes walks its list with a two-stage software prefetch: list entries
-// two ahead, partner data one ahead.  With frozen particles (FR = FORCE_ROUNDS)
-// a block gathers the mobile particles of several blocks' worth of slots and
-// runs them in rounds of 128, so its warps stay full instead of idling beside
-// the wall particles while they hold the block's resident slot.
+// two ahead, partner data one ahead.  With frozen particles in a large system
+// (FR = FORCE_ROUNDS, see frozen_rounds) a block gathers the mobile particles of
+// several blocks' worth of slots and runs them in rounds of 128, so its warps stay
+// full instead of idling beside the wall particles while they hold the block's
+// resident slot.
 // Minimum resident blocks per SM asked of the FP32 force kernel (0: the
 // compiler's default, kept for FP64).  The pair loop is latency-bound on its
 // partner gathers, so occupancy pays more than the few registers it costs: 8
@@ -151,9 +152,9 @@ k_force_nl(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt, MaskDev mk,
             const V* tP = tab.P + ti * 8;
             const uint32_t cnt = nl_count[s];
             // list column (see k_density_nl): the slot, or under list_compact
-            // (rounds blocks only) the block's first slot plus the place among
-            // its mobile particles, which the density pass formed the same way
-            const int64_t lcol = (FR > 1 && ph.list_compact)
+            // the block's first slot plus the place among its mobile particles,
+            // which the density pass formed the same way
+            const int64_t lcol = (!BATCH && LPP == 1 && ph.list_compact)
                                      ? (int64_t)blockIdx.x * (FR * PPB) + slot : (int64_t)s;
             if (cnt <= (uint32_t)NL_MAX) {
                 const uint32_t k0 = (uint32_t)sub;
@@ -302,7 +303,7 @@ void launch_force_nl_lpp(cudaStream_t st, ForceMode mode, int n, int64_t cap, co
         launch_force_nl_t<T, false, 2>(st, mode, n, cap, geo, ph, Batch{}, mk, pos4, vel4, rho,
                                        cell_s, start, nl, nl_count, step_ptr, step_offset, m, out,
                                        partials, status);
-    else if (force_nl_rounds(ph, 1) > 1)
+    else if (force_nl_rounds(ph, 1, n) > 1)
         launch_force_nl_t<T, false, 1, FORCE_ROUNDS>(st, mode, n, cap, geo, ph, Batch{}, mk, pos4,
                                                      vel4, rho, cell_s, start, nl, nl_count,
                                                      step_ptr, step_offset, m, out, partials,
@@ -315,7 +316,17 @@ void launch_force_nl_lpp(cudaStream_t st, ForceMode mode, int n, int64_t cap, co
 
 }  // namespace
 
-int force_nl_rounds(const Phys& ph, int lpp) { return lpp == 1 && ph.frozen ? FORCE_ROUNDS : 1; }
+// Rounds keep a block's warps full of mobile particles, but make a quarter of the
+// blocks: in a small system the chip is then nearly empty and a block's rounds are
+// its time.  Measured on porous rocks, density + force pass with 4 rounds and with 1:
+// 28k slots 119 and 57 us, 68k 110 and 58, 231k 126 and 107, 546k 181 and 199, 1.8M
+// 447 and 529.
+int frozen_rounds(int64_t n) { return n > 400000 ? FORCE_ROUNDS : 1; }
+
+int force_nl_rounds(const Phys& ph, int lpp, int64_t n)
+{
+    return lpp == 1 && ph.frozen ? frozen_rounds(n) : 1;
+}
 
 void launch_force_nl(cudaStream_t st, int precision, ForceMode mode, int n, int64_t cap,
                      const Geo& geo, const Phys& ph, int lpp, const MaskDev& mk, const void* pos4,

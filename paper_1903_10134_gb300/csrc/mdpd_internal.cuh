@@ -354,10 +354,14 @@ void launch_force(cudaStream_t st, int precision, ForceMode mode, int n, int64_t
 int force_num_blocks(int n, int lpp = 1, int rounds = 1);
 // Number of per-warp observable partials the force pass writes for n particles.
 int obs_num_partials(int n, int lpp = 1, int rounds = 1);
-// Rounds per block of the list force pass of a single system (FORCE_ROUNDS
-// with frozen particles at one lane per particle, else 1).
+// Rounds of a block of the density and force passes over n slots with frozen
+// particles: a block gathers the mobile particles of frozen_rounds(n) * PAIR_BLOCK
+// slots and runs them in rounds of PAIR_BLOCK (1 or FORCE_ROUNDS).
 constexpr int FORCE_ROUNDS = 4;
-int force_nl_rounds(const Phys& ph, int lpp);
+int frozen_rounds(int64_t n);
+// The same for the list force pass of a single system (1 without frozen particles
+// and at several lanes per particle).
+int force_nl_rounds(const Phys& ph, int lpp, int64_t n);
 // Density pass that also writes the force partners of mobile particles
 // (entries (j << 5) | image code, slot-major: nl[k * cap + column] with the
 // column of ph.list_compact; nl_count[i] by slot).
