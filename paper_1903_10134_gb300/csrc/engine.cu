@@ -1698,14 +1698,21 @@ void vjp_core(mdpd_handle* h, const double* abar, const double* wbar, const doub
     double* xs = h->x[1 - c];
     double* us = h->v[1 - c];
     double* rs = h->a[1 - c];
+    // partials of types a replica does not have are not formed: a batch with uneven
+    // ntypes starts from zero
+    int nt = h->nrep ? 0 : h->p.ntypes;
+    for (int r = 0; r < h->nrep; ++r) nt = std::max(nt, h->rep_p[r].ntypes);
+    bool even = true;
+    for (int r = 0; r < h->nrep; ++r) even = even && h->rep_p[r].ntypes == nt;
+    if (!even)
+        cudaMemsetAsync(h->vjp_tpart, 0, (size_t)vjp_num_blocks(n, pb) * THETA_SLOTS * sizeof(double), st);
     launch_force_vjp(st, h->precision, n, h->cap, h->geo, h->ph, pb, h->pos4, h->vel4, h->rho,
-                     h->cell_s, h->start, h->nl, h->nl_count, h->step, abar, wbar, xs, us, rs,
-                     h->vjp_tpart, h->status);
-    if (rhobar) launch_gather_by_id(st, n, h->id[c], rhobar, rs, 1);
+                     h->cell_s, h->start, h->nl, h->nl_count, h->step, h->id[c], abar, h->fout, wbar,
+                     rhobar, xs, us, rs, h->vjp_tpart, h->status);
     launch_density_vjp(st, h->precision, n, h->cap, h->geo, h->ph, pb, h->pos4, h->cell_s,
                        h->start, h->nl, h->nl_count, rs, xs, h->status);
     launch_theta_reduce(st, vjp_nrep(h), vjp_num_blocks(n, pb), h->nrep ? h->d_wr : nullptr,
-                        PAIR_BLOCK_WARPS, h->vjp_tpart, h->vjp_tacc, add_theta);
+                        PAIR_BLOCK_WARPS, nt, h->vjp_tpart, h->vjp_tacc, add_theta);
 }
 
 // Master state from device arrays in id order (no evaluation).

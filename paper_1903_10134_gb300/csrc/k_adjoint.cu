@@ -33,9 +33,9 @@
 //
 // Parameter gradients are deterministic: each thread accumulates its pairs'
 // terms in its own shared-memory column, indexed by (parameter, partner
-// type); the block then adds the columns of its threads in thread order for
+// type); the block then adds the columns of its threads by a fixed tree for
 // every (parameter, own type, partner type), and a per-replica kernel adds the
-// blocks in block order.  Each unordered pair is seen from both sides, so each
+// blocks in a fixed order.  Each unordered pair is seen from both sides, so each
 // side adds half its term.
 #include "pair.cuh"
 
@@ -45,6 +45,71 @@ namespace {
 
 constexpr int TB = 3 * 64;         // parameter slots [q][a][b], q = A, B, gamma
 constexpr int TCOL = 3 * 8;        // per-thread columns [q][partner type]
+
+// 1 / sqrt(x): FP32 from the hardware estimate (2 ulp) with one Newton step, FP64 by
+// the library function.  (Quotients by r are products with it: an FP64 division is
+// some ten instructions at 1/64 of the FP32 rate, and a pair had up to thirteen.)
+__device__ __forceinline__ float inv_sqrt(float x)
+{
+    const float y = rsqrtf(x);
+    return fmaf(0.5f * y, fmaf(-x * y, y, 1.0f), y);
+}
+__device__ __forceinline__ double inv_sqrt(double x) { return rsqrt(x); }
+// sqrt(x) from y = inv_sqrt(x): in FP32 with the rounding of x y taken back.
+__device__ __forceinline__ float sqrt_from(float x, float y)
+{
+    const float r = x * y;
+    return fmaf(0.5f * y, fmaf(-r, r, x), r);
+}
+__device__ __forceinline__ double sqrt_from(double x, double y) { return x * y; }
+
+// A parameter gradient's running sum over one particle's pairs.  In FP32 a pair of
+// floats (the rounding of every addition kept: Knuth's two-sum), as exact as the
+// FP64 sum and off the FP64 pipe.
+struct Sum2 {
+    float hi, lo;
+};
+template <typename T> struct ColSum;
+template <> struct ColSum<float> { using type = Sum2; };
+template <> struct ColSum<double> { using type = double; };
+__device__ __forceinline__ void col_add(Sum2& c, float x)
+{
+    const float s = __fadd_rn(c.hi, x), t = __fsub_rn(s, c.hi);
+    c.lo = __fadd_rn(c.lo, __fadd_rn(__fsub_rn(c.hi, __fsub_rn(s, t)), __fsub_rn(x, t)));
+    c.hi = s;
+}
+__device__ __forceinline__ void col_add(double& c, double x) { c += x; }
+__device__ __forceinline__ double col_value(const Sum2& c) { return (double)c.hi + (double)c.lo; }
+__device__ __forceinline__ double col_value(double c) { return c; }
+
+// Adjoints of the accelerations in cell order (zero for frozen particles): 16 bytes a
+// slot in FP32, 24 in FP64.
+__device__ __forceinline__ void store_abar(float4* a, int64_t s, double x, double y, double z)
+{
+    a[s] = make_float4((float)x, (float)y, (float)z, 0.0f);
+}
+__device__ __forceinline__ void store_abar(double* a, int64_t s, double x, double y, double z)
+{
+    a[3 * s] = x;
+    a[3 * s + 1] = y;
+    a[3 * s + 2] = z;
+}
+__device__ __forceinline__ void load_abar(const float4* __restrict__ a, int64_t s, float (&q)[3])
+{
+    const float4 v = a[s];
+    q[0] = v.x;
+    q[1] = v.y;
+    q[2] = v.z;
+}
+__device__ __forceinline__ void load_abar(const double* __restrict__ a, int64_t s, double (&q)[3])
+{
+    q[0] = a[3 * s];
+    q[1] = a[3 * s + 1];
+    q[2] = a[3 * s + 2];
+}
+template <typename T> struct AbarOf;
+template <> struct AbarOf<float> { using type = float4; };
+template <> struct AbarOf<double> { using type = double; };
 
 // The block's particle slot, replica record and validity (see Batch).
 template <bool BATCH>
@@ -123,6 +188,19 @@ __device__ __forceinline__ void for_partners(int s, uint32_t cnt, int64_t cap,
     }
 }
 
+// abar (id order) to cell order in the pair precision.
+template <typename T>
+__global__ void k_gather_abar(int n, const uint32_t* __restrict__ id, const double* __restrict__ abar, typename AbarOf<T>::type* __restrict__ out)
+{
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= n) return;
+    const int64_t i = id[s];
+    store_abar(out, s, abar[3 * i], abar[3 * i + 1], abar[3 * i + 2]);
+}
+
+// Bound by issue (FP32: about 130 instructions a pair, 45 of them the draw) and, in
+// FP64, by the FP64 pipe (70 a pair).  The parameters' sums per pair stay out of it:
+// tables in the pair precision, running sums in Sum2.
 template <typename T, bool BATCH>
 __global__ void __launch_bounds__(PAIR_BLOCK)
 k_force_vjp(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
@@ -130,36 +208,44 @@ k_force_vjp(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
             const typename Vec4<T>::type* __restrict__ vel4, const T* __restrict__ rho,
             const uint32_t* __restrict__ cell_s, const uint32_t* __restrict__ start,
             const uint32_t* __restrict__ nl, const uint32_t* __restrict__ nl_count,
-            const uint64_t* __restrict__ step_ptr, const double* __restrict__ abar,
-            const double* __restrict__ wbar, double* __restrict__ xbar,
-            double* __restrict__ ubar, double* __restrict__ rbar, double* __restrict__ tpart,
+            const uint64_t* __restrict__ step_ptr,
+            const typename AbarOf<T>::type* __restrict__ abar, const double* __restrict__ wbar,
+            const double* __restrict__ rhobar, double* __restrict__ xbar,
+            double* __restrict__ ubar, T* __restrict__ rbar, double* __restrict__ tpart,
             uint32_t* __restrict__ status)
 {
     using V = typename Vec4<T>::type;
-    __shared__ double col[PAIR_BLOCK][TCOL + 1];
-    __shared__ uint8_t ty[PAIR_BLOCK];
+    using Col = typename ColSum<T>::type;
+    __shared__ Col col[TCOL][PAIR_BLOCK];
     __shared__ T shift[27][3];
+    __shared__ PairTables<T> tab;              // A, B, gamma, sigma / sqrt(dt)
+    __shared__ T dsig[64];                     // d(sigma)/d(gamma) / sqrt(dt)
+    __shared__ double wsum[PAIR_BLOCK / 32];
     const BlockSite<BATCH> b = block_site<BATCH>(n, bt);
     const Phys& ph = BATCH ? b.rp->ph : ph_p;             // scalars (and tables if single)
     const Phys& tabs = BATCH ? bt.reps[b.r].ph : ph_p;    // per-type-pair tables
     const uint32_t id0 = BATCH ? b.rp->id0 : 0u;
+    const Derived<T>& dc = derived<T>(ph);
     const int tid = threadIdx.x;
+    const int nt = ph.ntypes;
 #pragma unroll
-    for (int k = 0; k < TCOL; ++k) col[tid][k] = 0.0;
+    for (int q = 0; q < 3; ++q)
+        for (int t = 0; t < nt; ++t) col[q * 8 + t][tid] = Col{};
+    for (int k = tid; k < 64; k += PAIR_BLOCK) {
+        tab.P[k] = make4((T)tabs.A[k], (T)tabs.B[k], (T)tabs.gamma[k], (T)tabs.sigma[k] * dc.inv_sqrt_dt);
+        dsig[k] = tabs.gamma[k] > 0.0 ? (T)(ph.kT / tabs.sigma[k]) * dc.inv_sqrt_dt : T(0);
+    }
     if (tid < 27) {
-        shift[tid][0] = (T)(tid % 3 - 1) * derived<T>(ph).h[0];
-        shift[tid][1] = (T)((tid / 3) % 3 - 1) * derived<T>(ph).h[1];
-        shift[tid][2] = (T)(tid / 9 - 1) * derived<T>(ph).h[2];
+        shift[tid][0] = (T)(tid % 3 - 1) * dc.h[0];
+        shift[tid][1] = (T)((tid / 3) % 3 - 1) * dc.h[1];
+        shift[tid][2] = (T)(tid / 9 - 1) * dc.h[2];
     }
     const int s = b.s;
-    ty[tid] = b.valid ? (uint8_t)type_of(pos4[s].w) : (uint8_t)0xFF;
+    uint32_t ti = 0xFFu;
     __syncthreads();
     if (b.valid) {
         const uint64_t step = *step_ptr;
-        const Derived<T>& dc = derived<T>(ph);
         const T inv_rc = dc.inv_rc, inv_rd = dc.inv_rd;
-        const T rd = (T)ph.rd;
-        const T inv_sqrt_dt = dc.inv_sqrt_dt;
         // virial weights of this replica (c_xx c_yy c_zz c_xy c_xz c_yz)
         T cw[6] = { T(0), T(0), T(0), T(0), T(0), T(0) };
         const bool vir = wbar != nullptr;
@@ -169,12 +255,11 @@ k_force_vjp(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
         const V pi = pos4[s];
         const V vi = vel4[s];
         const T rho_i = rho[s];
-        const uint32_t ti = type_of(pi.w), id_i = unpack_u32(vi.w);
+        const uint32_t id_i = unpack_u32(vi.w);
+        ti = type_of(pi.w);
         const bool mob_i = ((ph.frozen >> ti) & 1u) == 0u;
         T ai[3] = { T(0), T(0), T(0) };
-        if (abar && mob_i)
-#pragma unroll
-            for (int k = 0; k < 3; ++k) ai[k] = (T)abar[3 * (int64_t)(id0 + id_i) + k];
+        if (abar && mob_i) load_abar(abar, s, ai);
         T gx[3] = { T(0), T(0), T(0) }, gu[3] = { T(0), T(0), T(0) };
         T gr = T(0);
         // one partner j in the image of neighbour-cell code `code`
@@ -188,45 +273,58 @@ k_force_vjp(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
             const T dy = pi.y - shift[code][1] - pj.y;
             const T dz = pi.z - shift[code][2] - pj.z;
             const T r2 = dx * dx + dy * dy + dz * dz;
-            const T r = sqrt(r2);
-            const T ex = dx / r, ey = dy / r, ez = dz / r;
-            const T e3[3] = { ex, ey, ez };
+            const T rinv = inv_sqrt(r2);
+            const T r = sqrt_from(r2, rinv);
+            const T e3[3] = { dx * rinv, dy * rinv, dz * rinv };
             const T wc = T(1) - r * inv_rc;
-            const bool near = r < rd;
-            const T wd = near ? T(1) - r * inv_rd : T(0);
-            const int pidx = ti * 8 + tj;
-            const T A = (T)tabs.A[pidx], B = (T)tabs.B[pidx];
+            const T wd0 = T(1) - r * inv_rd;
+            const bool near = wd0 > T(0);
+            const T wd = near ? wd0 : T(0);
+            const int pidx = (int)(ti * 8 + tj);
+            const V prm = tab.P[pidx];
+            const T A = prm.x, B = prm.y;
             const T rsum = rho_i + rho_j;
-            double* cl = col[tid];
+            const T sc = A * wc + B * rsum * wd;                                // F^C
+            const T sc_r = -A * inv_rc - (near ? B * rsum * inv_rd : T(0));     // its d/dr
             if (abar) {
-                T q[3];
+                T q[3] = { T(0), T(0), T(0) };
+                if (mob_j) load_abar(abar, j, q);
 #pragma unroll
-                for (int c = 0; c < 3; ++c)
-                    q[c] = ai[c] - (mob_j ? (T)abar[3 * (int64_t)(id0 + id_j) + c] : T(0));
-                const T ux = vi.x - vj.x, uy = vi.y - vj.y, uz = vi.z - vj.z;
-                const T u3[3] = { ux, uy, uz };
-                const T w = ex * ux + ey * uy + ez * uz;
-                const T G = (T)tabs.gamma[pidx];
-                const T sig = (T)tabs.sigma[pidx];
-                const U4 wr = pair_draw(id_i, id_j, step, ph.key0, ph.key1);
+                for (int c = 0; c < 3; ++c) q[c] = ai[c] - q[c];
+                const T u3[3] = { vi.x - vj.x, vi.y - vj.y, vi.z - vj.z };
+                const T w = e3[0] * u3[0] + e3[1] * u3[1] + e3[2] * u3[2];
+                const U4 wr = BATCH ? pair_draw(id_i, id_j, step, ph.key0, ph.key1)
+                                    : pair_draw_rk(id_i, id_j, step, ph.rk);
                 const T xi = xi_of<T>(wr, ph.xi_dist);
-                const T sval = A * wc + B * rsum * wd - G * wc * wc * w + sig * wc * xi * inv_sqrt_dt;
-                const T s_r = -A * inv_rc - (near ? B * rsum * inv_rd : T(0)) +
-                              T(2) * G * wc * w * inv_rc - sig * xi * inv_sqrt_dt * inv_rc;
-                const T s_w = -G * wc * wc;
-                const T qe = q[0] * ex + q[1] * ey + q[2] * ez;
+                const T gw = prm.z * wc, sx = prm.w * xi;      // gamma wc, sigma xi / sqrt(dt)
+                const T sval = sc + wc * (sx - gw * w);
+                const T s_r = sc_r + (T(2) * gw * w - sx) * inv_rc;
+                const T s_w = -gw * wc;
+                const T qe = q[0] * e3[0] + q[1] * e3[1] + q[2] * e3[2];
+                const T be = qe * s_w, sr = sval * rinv, br = be * rinv;
+                if constexpr (sizeof(T) == 8) {
+                // (q.e) s_r e + br (u - w e) + sr (q - (q.e) e), by the vectors' sums
+                const T al = qe * (s_r - sr) - br * w;
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    gx[c] += qe * (s_r * e3[c] + s_w * (u3[c] - w * e3[c]) / r) +
-                             sval * (q[c] - qe * e3[c]) / r;
-                    gu[c] += qe * s_w * e3[c];
+                    gx[c] += al * e3[c];
+                    gx[c] += br * u3[c];
+                    gx[c] += sr * q[c];
+                    gu[c] += be * e3[c];
+                }
+                } else {
+                const T al = qe * s_r;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    gx[c] += al * e3[c] + br * (u3[c] - w * e3[c]) + sr * (q[c] - qe * e3[c]);
+                    gu[c] += be * e3[c];
+                }
                 }
                 gr += qe * B * wd;
-                const double dsig = tabs.gamma[pidx] > 0.0 ? ph.kT / tabs.sigma[pidx] : 0.0;
-                cl[0 * 8 + tj] += 0.5 * (double)(qe * wc);
-                cl[1 * 8 + tj] += 0.5 * (double)(qe * rsum * wd);
-                cl[2 * 8 + tj] += 0.5 * (double)(qe * (-wc * wc * w)) +
-                                  0.5 * (double)qe * dsig * (double)(wc * xi * inv_sqrt_dt);
+                const T hq = T(0.5) * qe;
+                col_add(col[tj][tid], hq * wc);
+                col_add(col[8 + tj][tid], hq * rsum * wd);
+                col_add(col[16 + tj][tid], hq * wc * (dsig[pidx] * xi - wc * w));
             }
             if (vir) {
                 const T mm = T((mob_i ? 1 : 0) + (mob_j ? 1 : 0));
@@ -236,39 +334,47 @@ k_force_vjp(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
                     const T gQ[3] = { T(2) * cw[0] * dx + cw[3] * dy + cw[4] * dz,
                                       T(2) * cw[1] * dy + cw[3] * dx + cw[5] * dz,
                                       T(2) * cw[2] * dz + cw[4] * dx + cw[5] * dy };
-                    const T sc = A * wc + B * rsum * wd;
-                    const T sc_r = -A * inv_rc - (near ? B * rsum * inv_rd : T(0));
-                    const T Qr = Q / r;
-                    const T d3[3] = { dx, dy, dz };
+                    const T hm = T(0.5) * mm, Qr = Q * rinv;
+                    const T sq = hm * sc * rinv, er = hm * Qr * (sc_r - sc * rinv);
 #pragma unroll
-                    for (int c = 0; c < 3; ++c)
-                        gx[c] += T(0.5) * mm *
-                                 (sc * (gQ[c] / r - Q * d3[c] / (r2 * r)) + Qr * sc_r * e3[c]);
-                    gr += T(0.5) * mm * Qr * B * wd;
-                    cl[0 * 8 + tj] += 0.25 * (double)(mm * Qr * wc);
-                    cl[1 * 8 + tj] += 0.25 * (double)(mm * Qr * rsum * wd);
+                    for (int c = 0; c < 3; ++c) gx[c] += sq * gQ[c] + er * e3[c];
+                    gr += hm * Qr * B * wd;
+                    const T hr = T(0.5) * hm * Qr;
+                    col_add(col[tj][tid], hr * wc);
+                    col_add(col[8 + tj][tid], hr * rsum * wd);
                 }
             }
         };
         const Geo& geo = BATCH ? b.rp->geo : geo_p;
-        for_partners<T>(s, nl_count[s], cap, nl, geo, BATCH ? b.rp->cell0 : 0, cell_s, start, pos4,
-                        pi, shift, derived<T>(ph).rc2, ph.dbg_status, partner);
+        if (abar || vir)
+            for_partners<T>(s, nl_count[s], cap, nl, geo, BATCH ? b.rp->cell0 : 0, cell_s, start, pos4,
+                            pi, shift, derived<T>(ph).rc2, ph.dbg_status, partner);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             xbar[c * cap + s] = (double)gx[c];
             ubar[c * cap + s] = (double)gu[c];
         }
-        rbar[s] = (double)gr;
+        rbar[s] = rhobar ? (T)((double)gr + rhobar[id0 + id_i]) : gr;
     }
-    __syncthreads();
-    // slot (q, a, b): the columns (q, b) of the block's threads of type a, in
-    // thread order
-    for (int k = tid; k < TB; k += PAIR_BLOCK) {
+    // slot (q, a, b): the columns (q, b) of the block's threads of type a, added over
+    // the warp by a fixed tree and over the warps in order
+    const int lane = tid & 31, warp = tid >> 5;
+    for (int k = 0; k < TB; ++k) {
         const int q = k / 64, a = (k / 8) % 8, bb = k % 8;
-        double acc = 0.0;
-        for (int t = 0; t < PAIR_BLOCK; ++t)
-            if (ty[t] == a) acc += col[t][q * 8 + bb];
-        tpart[(int64_t)blockIdx.x * TB + k] = acc;
+        double v = 0.0;
+        if (a < nt && bb < nt) {                          // (block-uniform)
+            if (ti == (uint32_t)a) v = col_value(col[q * 8 + bb][tid]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            __syncthreads();
+            if (lane == 0) wsum[warp] = v;
+            __syncthreads();
+            if (tid == 0) {
+                v = wsum[0];
+                for (int t = 1; t < PAIR_BLOCK / 32; ++t) v += wsum[t];
+                tpart[(int64_t)blockIdx.x * TB + k] = v;
+            }
+        }
     }
 }
 
@@ -278,7 +384,7 @@ k_density_vjp(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
               const typename Vec4<T>::type* __restrict__ pos4,
               const uint32_t* __restrict__ cell_s, const uint32_t* __restrict__ start,
               const uint32_t* __restrict__ nl, const uint32_t* __restrict__ nl_count,
-              const double* __restrict__ rbar, double* __restrict__ xbar,
+              const T* __restrict__ rbar, double* __restrict__ xbar,
               uint32_t* __restrict__ status)
 {
     using V = typename Vec4<T>::type;
@@ -295,20 +401,20 @@ k_density_vjp(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
     if (!b.valid) return;
     const int s = b.s;
     const Derived<T>& dc = derived<T>(ph);
-    const T rd = (T)ph.rd, inv_rd = dc.inv_rd;
-    const T cw = dc.cw_rho;
+    const T inv_rd = dc.inv_rd;
+    const T cw = T(-2) * dc.cw_rho * inv_rd;              // w_rho'(r) = cw (1 - r / r_d)
     const V pi = pos4[s];
-    const T rb_i = (T)rbar[s];
+    const T rb_i = rbar[s];
     T g[3] = { T(0), T(0), T(0) };
     auto partner = [&](uint32_t j, uint32_t code) {
         const V pj = pos4[j];
         const T dx = pi.x - shift[code][0] - pj.x;
         const T dy = pi.y - shift[code][1] - pj.y;
         const T dz = pi.z - shift[code][2] - pj.z;
-        const T r = sqrt(dx * dx + dy * dy + dz * dz);
-        if (!(r < rd)) return;
-        const T dw = T(-2) * cw * (T(1) - r * inv_rd) * inv_rd;   // w_rho'(r)
-        const T f = (rb_i + (T)rbar[j]) * dw / r;
+        const T r2 = dx * dx + dy * dy + dz * dz;
+        if (!(r2 < dc.rd2)) return;
+        const T rinv = inv_sqrt(r2);
+        const T f = (rb_i + rbar[j]) * cw * (rinv - inv_rd);      // ... w_rho'(r) / r
         g[0] += f * dx;
         g[1] += f * dy;
         g[2] += f * dz;
@@ -320,31 +426,49 @@ k_density_vjp(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
     for (int c = 0; c < 3; ++c) xbar[c * cap + s] += (double)g[c];
 }
 
-// rbar in cell order from the caller's rhobar in id order (stored, or added
-// to what the force VJP left there).
-__global__ void k_gather_by_id(int n, const uint32_t* __restrict__ id,
-                               const double* __restrict__ in, double* __restrict__ out, int add)
-{
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < n) out[s] = add ? out[s] + in[id[s]] : in[id[s]];
-}
-
-// Per replica (one block each, TB threads): the sum of its blocks' parameter
-// partials in block order, stored (add = 0) or added (add = 1) to acc.
+// Per replica (one block each): the sum of its blocks' parameter partials, stored
+// (add = 0) or added (add = 1) to acc.  P warps take a slot: their lanes add every
+// 32 P-th block and are added by a fixed tree, then the warps in order.  Only slots of
+// types below nt are formed (the others are zero).  (One thread per slot added the
+// blocks one after another: 99 us for 782 blocks.)
 // ranges[r] = (first, end) of replica r's blocks (x4 for warp ranges: scale).
-__global__ void k_theta_reduce(int nrep, int nblk, const int2* __restrict__ ranges, int scale,
-                               const double* __restrict__ tpart, double* __restrict__ acc, int add)
+constexpr int RED_WARPS = 32;
+__global__ void __launch_bounds__(RED_WARPS * 32)
+k_theta_reduce(int nrep, int nblk, const int2* __restrict__ ranges, int scale, int nt,
+               const double* __restrict__ tpart, double* __restrict__ acc, int add)
 {
-    const int r = blockIdx.x, k = threadIdx.x;
-    if (r >= nrep || k >= TB) return;
+    const int r = blockIdx.x, lane = threadIdx.x & 31;
     int lo = 0, hi = nblk;
     if (ranges) {
         lo = ranges[r].x / scale;
         hi = ranges[r].y / scale;
     }
-    double sum = 0.0;
-    for (int b = lo; b < hi; ++b) sum += tpart[(int64_t)b * TB + k];
-    acc[(int64_t)r * TB + k] = add ? acc[(int64_t)r * TB + k] + sum : sum;
+    __shared__ double part[RED_WARPS];
+    const int warp = threadIdx.x >> 5;
+    const int used = 3 * nt * nt;
+    const int P = max(1, RED_WARPS / used), S = RED_WARPS / P;      // warps a slot, slots at once
+    for (int u0 = 0; u0 < used; u0 += S) {
+        const int u = u0 + warp / P, p = warp % P;
+        const bool on = warp < S * P && u < used;
+        const int k = on ? u / (nt * nt) * 64 + u / nt % nt * 8 + u % nt : 0;
+        double sum = 0.0;
+        if (on) {
+#pragma unroll 4
+            for (int b = lo + 32 * p + lane; b < hi; b += 32 * P) sum += tpart[(int64_t)b * TB + k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+            if (lane == 0) part[warp] = sum;
+        }
+        __syncthreads();
+        if (on && p == 0 && lane == 0) {
+            for (int t = 1; t < P; ++t) sum += part[warp + t];
+            acc[(int64_t)r * TB + k] = add ? acc[(int64_t)r * TB + k] + sum : sum;
+        }
+        __syncthreads();
+    }
+    if (!add)
+        for (int k = threadIdx.x; k < TB; k += RED_WARPS * 32)
+            if ((k / 8) % 8 >= nt || k % 8 >= nt) acc[(int64_t)r * TB + k] = 0.0;
 }
 
 // Gradient of the symmetric tables from the per-(own type, partner type) sums
@@ -487,57 +611,46 @@ void launch_force_vjp(cudaStream_t st, int precision, int n, int64_t cap, const 
                       const Phys& ph, const Batch* bt, const void* pos4, const void* vel4,
                       const void* rho, const uint32_t* cell_s, const uint32_t* start,
                       const uint32_t* nl, const uint32_t* nl_count, const uint64_t* step_ptr,
-                      const double* abar, const double* wbar, double* xbar, double* ubar,
-                      double* rbar, double* tpart, uint32_t* status)
+                      const uint32_t* id, const double* abar, void* abar_s, const double* wbar,
+                      const double* rhobar, double* xbar, double* ubar, void* rbar, double* tpart,
+                      uint32_t* status)
 {
     const int nb = vjp_num_blocks(n, bt);
     if (nb <= 0) return;
     const Batch bb = bt ? *bt : Batch{};
     const size_t smem = bt ? REP_SMEM : 0;
-#define MDPD_FVJP(T_, B_)                                                                       \
-    k_force_vjp<T_, B_><<<nb, PAIR_BLOCK, smem, st>>>(                                        \
-        n, cap, geo, ph, bb, (const typename Vec4<T_>::type*)pos4,                                \
-        (const typename Vec4<T_>::type*)vel4, (const T_*)rho, cell_s, start, nl, nl_count,        \
-        step_ptr, abar, wbar, xbar, ubar, rbar, tpart, status)
-    if (precision == 0) {
-        if (bt) MDPD_FVJP(double, true);
-        else MDPD_FVJP(double, false);
-    } else {
-        if (bt) MDPD_FVJP(float, true);
-        else MDPD_FVJP(float, false);
-    }
-#undef MDPD_FVJP
+    auto go = [&](auto t, auto k) {
+        using T = decltype(t);
+        using A = typename AbarOf<T>::type;
+        using V = typename Vec4<T>::type;
+        if (abar)
+            k_gather_abar<T><<<(n + 255) / 256, 256, 0, st>>>(n, id, abar, (A*)abar_s);
+        k<<<nb, PAIR_BLOCK, smem, st>>>(n, cap, geo, ph, bb, (const V*)pos4, (const V*)vel4,
+                                        (const T*)rho, cell_s, start, nl, nl_count, step_ptr,
+                                        abar ? (const A*)abar_s : nullptr, wbar, rhobar, xbar, ubar,
+                                        (T*)rbar, tpart, status);
+    };
+    if (precision == 0) go(double{}, bt ? k_force_vjp<double, true> : k_force_vjp<double, false>);
+    else go(float{}, bt ? k_force_vjp<float, true> : k_force_vjp<float, false>);
 }
 
 void launch_density_vjp(cudaStream_t st, int precision, int n, int64_t cap, const Geo& geo,
                         const Phys& ph, const Batch* bt, const void* pos4,
                         const uint32_t* cell_s, const uint32_t* start, const uint32_t* nl,
-                        const uint32_t* nl_count, const double* rbar, double* xbar,
+                        const uint32_t* nl_count, const void* rbar, double* xbar,
                         uint32_t* status)
 {
     const int nb = vjp_num_blocks(n, bt);
     if (nb <= 0) return;
     const Batch bb = bt ? *bt : Batch{};
     const size_t smem = bt ? REP_SMEM : 0;
-#define MDPD_DVJP(T_, B_)                                                                       \
-    k_density_vjp<T_, B_><<<nb, PAIR_BLOCK, smem, st>>>(                                      \
-        n, cap, geo, ph, bb, (const typename Vec4<T_>::type*)pos4, cell_s, start, nl, nl_count,  \
-        rbar, xbar, status)
-    if (precision == 0) {
-        if (bt) MDPD_DVJP(double, true);
-        else MDPD_DVJP(double, false);
-    } else {
-        if (bt) MDPD_DVJP(float, true);
-        else MDPD_DVJP(float, false);
-    }
-#undef MDPD_DVJP
-}
-
-void launch_gather_by_id(cudaStream_t st, int n, const uint32_t* id, const double* in, double* out,
-                         int add)
-{
-    if (n <= 0) return;
-    k_gather_by_id<<<pair_blocks(n), PAIR_BLOCK, 0, st>>>(n, id, in, out, add);
+    auto go = [&](auto t, auto k) {
+        using T = decltype(t);
+        k<<<nb, PAIR_BLOCK, smem, st>>>(n, cap, geo, ph, bb, (const typename Vec4<T>::type*)pos4,
+                                        cell_s, start, nl, nl_count, (const T*)rbar, xbar, status);
+    };
+    if (precision == 0) go(double{}, bt ? k_density_vjp<double, true> : k_density_vjp<double, false>);
+    else go(float{}, bt ? k_density_vjp<float, true> : k_density_vjp<float, false>);
 }
 
 __global__ void k_set_u64(uint64_t* __restrict__ p, uint64_t v) { *p = v; }
@@ -548,10 +661,10 @@ void launch_set_step(cudaStream_t st, uint64_t* step_ptr, uint64_t value)
 }
 
 void launch_theta_reduce(cudaStream_t st, int nrep, int nblk, const int2* ranges, int scale,
-                         const double* tpart, double* acc, int add)
+                         int nt, const double* tpart, double* acc, int add)
 {
     if (nrep <= 0) return;
-    k_theta_reduce<<<nrep, TB, 0, st>>>(nrep, nblk, ranges, scale, tpart, acc, add);
+    k_theta_reduce<<<nrep, RED_WARPS * 32, 0, st>>>(nrep, nblk, ranges, scale, nt, tpart, acc, add);
 }
 
 void launch_theta_symmetrise(cudaStream_t st, int nrep, const double* acc, double* out)

@@ -85,9 +85,7 @@ k_frozen_part(int n, int64_t cap, Geo geo, Phys ph, const typename Vec4<T>::type
     }
     int q0, q1, q2;
     cell_coords(cell_s[s], geo, q0, q1, q2);
-    // the scan meets the home itself (r = 0, weight w(0)); that term is taken
-    // off at the end unless the self term is asked for
-    T acc = T(0);
+    T acc = ph.rho_self ? dc.cw_rho : T(0);
     for (int oz = -1; oz <= 1; ++oz) {
         const int z = neighbour_index(q2, oz, geo.nc[2], geo.periodic[2]);
         if (z < 0) continue;
@@ -107,7 +105,7 @@ k_frozen_part(int n, int64_t cap, Geo geo, Phys ph, const typename Vec4<T>::type
                     const auto pj = pos4[j];
                     const T dx = sx - pj.x, dy = sy - pj.y, dz = sz - pj.z;
                     const T r2 = dx * dx + dy * dy + dz * dz;
-                    if (r2 < dc.rc2 && ((ph.frozen >> type_of(pj.w)) & 1u)) {
+                    if (r2 < dc.rc2 && ((ph.frozen >> type_of(pj.w)) & 1u) && j != (uint32_t)s) {
                         const T w = max(T(1) - sqrt_fast(r2) * dc.inv_rd, T(0));
                         const T term = dc.cw_rho * w * w;      // r = 0 gives w(0)
                         acc += term;
@@ -116,7 +114,6 @@ k_frozen_part(int n, int64_t cap, Geo geo, Phys ph, const typename Vec4<T>::type
             }
         }
     }
-    if (!ph.rho_self) acc -= dc.cw_rho;
     rho_ff[id_s[s]] = acc;
 }
 
@@ -277,9 +274,7 @@ __device__ __forceinline__ void density_home(
     // wall density of a mobile particle (WANT_PHI): sum over frozen partners
     // within r_c of 15/(2 pi r_c^3) (1 - r/r_c)^2
     const bool want_phi = WANT_PHI && mob_true;
-    // the scan meets the home itself (r = 0, weight w(0)); that term is taken
-    // off at the end unless the self term is asked for
-    T acc = T(0), phi = T(0);
+    T acc = ph.rho_self ? dc.cw_rho : T(0), phi = T(0);
     uint32_t cnt = 0;
     uint32_t* lp = nl + lcol;                   // next list entry: nl[cnt * cap + lcol]
     // cell column of a candidate across a periodic face, from the home's
@@ -345,6 +340,10 @@ __device__ __forceinline__ void density_home(
                                __hfma2(dz1, dz1, __hfma2(dy1, dy1, __hfma2(dx1, dx1, thr))));
             }
             m = (m >> ((0u - k1) & 3u)) << (32u - k1) & (0xffffffffu >> lead);
+            // not the home itself: its own term is left out of the sum rather than
+            // taken off it (it is the largest, and the sum's rounding would grow)
+            const uint32_t self = (uint32_t)s - (rb & 0x07ffffffu);
+            if (self < 32u) m &= ~(0x80000000u >> self);
             if (m) {
                 sm.a[nw][tid] = m;
                 sm.b[nw][tid] = rb;
@@ -419,7 +418,7 @@ __device__ __forceinline__ void density_home(
                     const bool fz = (FS == 1 || WANT_PHI) && ((ph.frozen >> (bits & 7u)) & 1u);
                     if (FS == 1 && fz && term > 0.0f && pass == 0)
                         atomicAdd(facc + (jr & 0x07ffffffu), to_fixed(term * dc.fix_scale));
-                    if (mobile && r2 > 0.0f) {      // not the home, not coincident
+                    if (mobile && r2 > 0.0f) {      // not coincident
                         append(jr, code);
                         if (want_phi && fz && pass == 0) {
                             const float wq = 1.0f - sqrt_t(r2) * dc.inv_rc;
@@ -527,7 +526,6 @@ __device__ __forceinline__ void density_home(
     }
     }
     if (sub != 0) return;
-    if (!ph.rho_self) acc = rho_add(acc, -dc.cw_rho);
     rho_out[s] = acc;
     nl_count[s] = cnt;
     if (WANT_PHI) ((T*)ph.phi_out)[s] = phi;

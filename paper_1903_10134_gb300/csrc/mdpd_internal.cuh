@@ -52,6 +52,7 @@ struct Derived {
     T cw_rho;        // 15 / (2 pi r_d^3): density weight normalisation (Sec. 2.1)
     T cw_phi;        // 15 / (2 pi r_c^3): wall-density weight normalisation
     T inv_sqrt_dt;   // random force scale 1 / sqrt(dt)
+    T xi_scale;      // the same times sqrt(3) 2^-24 for the uniform draw (PairTables)
     T h[3];          // cell edges
     T hdt;           // dt / 2
     T g[3];          // body force
@@ -105,6 +106,7 @@ inline void fill_derived(Phys& ph, const Geo& geo)
     d.cw_rho = 15.0 / (2.0 * pi * ph.rd * ph.rd * ph.rd);
     d.cw_phi = 15.0 / (2.0 * pi * ph.rc * ph.rc * ph.rc);
     d.inv_sqrt_dt = ph.dt > 0.0 ? 1.0 / std::sqrt(ph.dt) : 0.0;
+    d.xi_scale = ph.xi_dist == 0 ? std::ldexp(std::sqrt(3.0), -24) * d.inv_sqrt_dt : d.inv_sqrt_dt;
     for (int k = 0; k < 3; ++k) d.h[k] = geo.h[k];
     d.hdt = 0.5 * ph.dt;
     ph.fast_cell = 0;
@@ -134,6 +136,7 @@ inline void fill_derived(Phys& ph, const Geo& geo)
     f.cw_rho = (float)d.cw_rho;
     f.cw_phi = (float)d.cw_phi;
     f.inv_sqrt_dt = (float)d.inv_sqrt_dt;
+    f.xi_scale = (float)d.xi_scale;
     for (int k = 0; k < 3; ++k) f.h[k] = (float)d.h[k];
     f.hdt = (float)d.hdt;
     for (int k = 0; k < 3; ++k) {
@@ -423,31 +426,34 @@ void launch_reduce_obs_batch(cudaStream_t st, int precision, const double* parti
 int vjp_num_blocks(int n, const Batch* bt);
 // VJP of one force evaluation at the current cell-ordered state (lists built
 // with list_all): abar (id order, may be NULL) the adjoint of the
-// accelerations, wbar (6 per replica, may be NULL) weights of the virial
-// components; xbar, ubar, rbar outputs in cell order; tpart[block][3 * 64]
-// the blocks' parameter partials by (parameter, own type, partner type).
+// accelerations (put in cell order in abar_s, 24 bytes a slot), wbar (6 per
+// replica, may be NULL) weights of the virial components, rhobar (id order, may be
+// NULL) the caller's adjoint of the densities; xbar, ubar outputs in cell order;
+// rbar (pair precision, cell order) the adjoint of the densities, rhobar included;
+// tpart[block][3 * 64] the blocks' parameter partials by (parameter, own type,
+// partner type), of types below the replica's ntypes only.
 void launch_force_vjp(cudaStream_t st, int precision, int n, int64_t cap, const Geo& geo,
                       const Phys& ph, const Batch* bt, const void* pos4, const void* vel4,
                       const void* rho, const uint32_t* cell_s, const uint32_t* start,
                       const uint32_t* nl, const uint32_t* nl_count, const uint64_t* step_ptr,
-                      const double* abar, const double* wbar, double* xbar, double* ubar,
-                      double* rbar, double* tpart, uint32_t* status);
+                      const uint32_t* id, const double* abar, void* abar_s, const double* wbar,
+                      const double* rhobar, double* xbar, double* ubar, void* rbar, double* tpart,
+                      uint32_t* status);
 // The density chain: xbar (cell order, [3][cap]) += sum_j (rbar_i + rbar_j)
-// w_rho'(r) e over partners within r_d (rbar in cell order).
+// w_rho'(r) e over partners within r_d (rbar as left by launch_force_vjp).
 void launch_density_vjp(cudaStream_t st, int precision, int n, int64_t cap, const Geo& geo,
                         const Phys& ph, const Batch* bt, const void* pos4,
                         const uint32_t* cell_s, const uint32_t* start, const uint32_t* nl,
-                        const uint32_t* nl_count, const double* rbar, double* xbar,
+                        const uint32_t* nl_count, const void* rbar, double* xbar,
                         uint32_t* status);
-void launch_gather_by_id(cudaStream_t st, int n, const uint32_t* id, const double* in, double* out,
-                         int add);
 // *step_ptr = value, ordered on the stream.
 void launch_set_step(cudaStream_t st, uint64_t* step_ptr, uint64_t value);
 constexpr int THETA_SLOTS = 3 * 64;   // [parameter][type][type] of A, B, gamma
-// Per replica: acc[r] (= or +=) the sum of its blocks' partials in block
-// order; ranges[r] / scale = the replica's block range (NULL: all nblk).
+// Per replica: acc[r] (= or +=) the sum of its blocks' partials in a fixed order, for
+// types below nt (0 for the others); ranges[r] / scale = the replica's block range
+// (NULL: all nblk).
 void launch_theta_reduce(cudaStream_t st, int nrep, int nblk, const int2* ranges, int scale,
-                         const double* tpart, double* acc, int add);
+                         int nt, const double* tpart, double* acc, int add);
 // Symmetric-table gradient [r][3][8][8] from the per-type-pair sums.
 void launch_theta_symmetrise(cudaStream_t st, int nrep, const double* acc, double* out);
 // Window checkpoints, start of the reverse sweep, and one reverse step's

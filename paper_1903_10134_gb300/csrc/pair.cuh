@@ -16,7 +16,7 @@ constexpr int NOBS = 14;     // momentum 3, sum v^2 3, virial 6, mobile count 1,
 constexpr int NL_MAX = NL_SLOTS;   // neighbour-list slots per particle (more: direct scan)
 
 __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrt_t(double x) { return 1.0 / sqrt(x); }
+__device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
 // r from r^2 (> 0) for the density weight: FP32 through the hardware reciprocal
 // square root (about 2 ulp), FP64 correctly rounded.
 __device__ __forceinline__ float sqrt_t(float x) { return x * rsqrtf(x); }
@@ -35,6 +35,15 @@ __device__ __forceinline__ float sqrt_fast(float x)
 }
 __device__ __forceinline__ double sqrt_fast(double x) { return sqrt(x); }
 
+// The draw that the tables' random scale multiplies: the uniform's integer, or xi.
+template <typename T>
+__device__ __forceinline__ T draw_of(U4 w, int dist)
+{
+    if (dist == 0) return (T)xi_uniform_int(w.x);
+    if constexpr (sizeof(T) == 4) return xi_gauss_f(w.x, w.y);
+    else return xi_gauss_d(w.x, w.y);
+}
+
 template <typename T>
 __device__ __forceinline__ T xi_of(U4 w, int dist)
 {
@@ -43,25 +52,28 @@ __device__ __forceinline__ T xi_of(U4 w, int dist)
     else return xi_gauss_d(w.x, w.y);
 }
 
-// Per-type-pair tables in shared memory, row ti: A, B, gamma, sigma.
+// Per-type-pair tables in shared memory, row ti: A, B, gamma and the random force's
+// scale sigma / sqrt(dt), times sqrt(3) 2^-24 for the uniform draw, whose integer m
+// (xi = sqrt(3) m 2^-24) it multiplies.
 template <typename T>
 struct PairTables {
-    typename Vec4<T>::type P[64];     // (A, B, gamma, sigma) of type pair [ti * 8 + tj]
+    typename Vec4<T>::type P[64];     // of type pair [ti * 8 + tj]
 };
 
 template <typename T>
 __device__ __forceinline__ void load_tables(PairTables<T>& t, const Phys& ph)
 {
     for (int k = threadIdx.x; k < 64; k += blockDim.x)
-        t.P[k] = make4((T)ph.A[k], (T)ph.B[k], (T)ph.gamma[k], (T)ph.sigma[k]);
+        t.P[k] = make4((T)ph.A[k], (T)ph.B[k], (T)ph.gamma[k],
+                       (T)ph.sigma[k] * derived<T>(ph).xi_scale);
 }
 
 template <typename T>
 struct PairConst {
-    T rc2, rd2, inv_rc, inv_rd, inv_sqrt_dt;
+    T rc2, rd2, inv_rc, inv_rd;
     __device__ explicit PairConst(const Phys& ph)
         : rc2(derived<T>(ph).rc2), rd2(derived<T>(ph).rd2), inv_rc(derived<T>(ph).inv_rc),
-          inv_rd(derived<T>(ph).inv_rd), inv_sqrt_dt(derived<T>(ph).inv_sqrt_dt)
+          inv_rd(derived<T>(ph).inv_rd)
     {
     }
 };
@@ -76,18 +88,18 @@ __device__ __forceinline__ void pair_term(const PairConst<T>& c, const V4& prm, 
                                           uint32_t id_i, uint32_t id_j, uint64_t step,
                                           const Phys& ph, T (&f)[3], T (&W)[6])
 {
-    // prm = (A, B, gamma, sigma) of the pair's types
+    // prm = (A, B, gamma, random scale) of the pair's types
     const T rinv = rsqrt_t(r2);
     const T r = r2 * rinv;
     const T wc = T(1) - r * c.inv_rc;
     T fc = prm.x * wc;
     if (r2 < c.rd2) fc += prm.y * (rho_i + rho_j) * (T(1) - r * c.inv_rd);
     const T ev = (dx * (vi.x - vj.x) + dy * (vi.y - vj.y) + dz * (vi.z - vj.z)) * rinv;
-    const T fd = -prm.z * wc * wc * ev;
     const U4 w = RK ? pair_draw_rk(id_i, id_j, step, ph.rk)
                     : pair_draw(id_i, id_j, step, ph.key0, ph.key1);
-    const T fr = prm.w * wc * xi_of<T>(w, ph.xi_dist) * c.inv_sqrt_dt;
-    const T fp = (fc + fd + fr) * rinv;
+    // F^D + F^R = w_C (random scale * draw - gamma w_C (e.v_ij))
+    const T fdr = prm.w * draw_of<T>(w, ph.xi_dist) - prm.z * wc * ev;
+    const T fp = (fc + wc * fdr) * rinv;
     f[0] += fp * dx;
     f[1] += fp * dy;
     f[2] += fp * dz;

@@ -94,10 +94,14 @@ __device__ __forceinline__ U4 pair_draw_rk(uint32_t id_i, uint32_t id_j, uint64_
 // Uniform xi with zero mean and unit variance: sqrt(3) * m * 2^-24 with the odd
 // integer m = 2 (w >> 8) + 1 - 2^24, exact in FP32 and FP64 before the
 // multiplication by sqrt(3).
+__device__ __forceinline__ int32_t xi_uniform_int(uint32_t w)
+{
+    return (int32_t)((w >> 8) << 1) + 1 - (1 << 24);
+}
 template <typename T>
 __device__ __forceinline__ T xi_uniform(uint32_t w)
 {
-    const int32_t m = (int32_t)((w >> 8) << 1) + 1 - (1 << 24);
+    const int32_t m = xi_uniform_int(w);
     return (T)1.7320508075688772935274463415059 * ((T)m * (T)5.9604644775390625e-8);
 }
 
