@@ -33,21 +33,14 @@ def _is_batch(system) -> bool:
 
 
 def _set_tables(system, params, A, B, G):
-    """Write the tables A, B, gamma into the handle's parameters."""
+    """Write the tables A, B, gamma into the handle's parameters (one copy of
+    each to the host, for all replicas of a batch)."""
+    tabs = [t.detach().double().cpu().numpy() for t in (A, B, G)]
     if _is_batch(system):
-        ps = []
-        for r, p in enumerate(params):
-            q = p.copy()
-            q.A = A[r].detach().double().cpu().numpy().copy()
-            q.B = B[r].detach().double().cpu().numpy().copy()
-            q.gamma = G[r].detach().double().cpu().numpy().copy()
-            ps.append(q)
-        M.mdpd_batch_set_params(system.h, ps)
+        M.mdpd_batch_set_params(system.h, params, [t[:len(params)] for t in tabs])
     else:
         q = params.copy()
-        q.A = A.detach().double().cpu().numpy().copy()
-        q.B = B.detach().double().cpu().numpy().copy()
-        q.gamma = G.detach().double().cpu().numpy().copy()
+        q.A, q.B, q.gamma = (t.copy() for t in tabs)
         M.mdpd_set_params(system.h, q)
 
 

@@ -67,9 +67,22 @@ class Params(C.Structure):
     ]
 
 
-def to_c_params(p) -> Params:
-    """Fill ``mdpd_params`` from any object with MDPDParams' attributes."""
-    c = Params()
+_PARAMS_DTYPE = np.dtype(Params)
+_TABLES = ("A", "B", "gamma")
+
+
+def _table(t) -> np.ndarray:
+    """The 8 x 8 corner of a pair table (any nested sequence of numbers)."""
+    try:
+        a = np.asarray(t, dtype=np.float64)
+        if a.ndim == 2 and min(a.shape) >= MAX_TYPES:
+            return a[:MAX_TYPES, :MAX_TYPES]
+    except (TypeError, ValueError):
+        pass
+    return np.array([[float(t[a][b]) for b in range(MAX_TYPES)] for a in range(MAX_TYPES)])
+
+
+def _fill_scalars(c: Params, p):
     for k in range(3):
         c.box_lo[k] = float(p.box_lo[k])
         c.box[k] = float(p.box[k])
@@ -77,16 +90,33 @@ def to_c_params(p) -> Params:
         c.g[k] = float(p.g[k])
     c.ntypes = int(p.ntypes)
     c.rc, c.rd, c.dt, c.kT = float(p.rc), float(p.rd), float(p.dt), float(p.kT)
-    for a in range(MAX_TYPES):
-        for b in range(MAX_TYPES):
-            c.A[a][b] = float(p.A[a][b])
-            c.B[a][b] = float(p.B[a][b])
-            c.gamma[a][b] = float(p.gamma[a][b])
     c.frozen_type_mask = int(p.frozen_mask)
     c.precision = int(p.precision)
     c.xi_dist = int(p.xi_dist)
     c.rho_self = int(p.rho_self)
-    return c
+
+
+def to_c_params(p) -> Params:
+    """Fill ``mdpd_params`` from any object with MDPDParams' attributes."""
+    return _c_params_list([p])[0]
+
+
+def _c_params_list(params_list, tables=None):
+    """Array of ``mdpd_params``; `tables` = (A, B, gamma), each (len, 8, 8), in
+    place of the objects' own."""
+    cps = (Params * len(params_list))()
+    if not len(params_list):
+        return cps
+    view = np.frombuffer(cps, dtype=_PARAMS_DTYPE)      # writes go to cps
+    for r, p in enumerate(params_list):
+        _fill_scalars(cps[r], p)
+        if tables is None:
+            for name in _TABLES:
+                view[name][r] = _table(getattr(p, name))
+    if tables is not None:
+        for name, t in zip(_TABLES, tables):
+            view[name][:] = t
+    return cps
 
 
 SYMBOLS = (
@@ -239,7 +269,7 @@ def mdpd_create_batch(params_list, n_list, pos, vel, type, seeds, stream=None):
     pos = _arr(pos, np.float64, (N, 3))
     vel = _arr(vel, np.float64, (N, 3))
     typ = _arr(type, np.int32, (N,))
-    cps = (Params * nrep)(*[to_c_params(p) for p in params_list])
+    cps = _c_params_list(params_list)
     sd = _arr([int(v) for v in seeds], np.uint64, (nrep,))
     h = C.c_void_p()
     _check(lib().mdpd_create_batch(nrep, cps, _p(ns), _p(pos), _p(vel), _p(typ), _p(sd),
@@ -259,8 +289,9 @@ def mdpd_batch_observables(h, mean: bool = False, reset: bool = False) -> np.nda
     return out
 
 
-def mdpd_batch_set_params(h, params_list):
-    cps = (Params * len(params_list))(*[to_c_params(p) for p in params_list])
+def mdpd_batch_set_params(h, params_list, tables=None):
+    """`tables` = (A, B, gamma), each (nrep, 8, 8), in place of the objects' own."""
+    cps = _c_params_list(params_list, tables)
     _check(lib().mdpd_batch_set_params(h, cps), h)
 
 
