@@ -394,7 +394,7 @@ int mdpd_describe(const mdpd_handle* h, int32_t ncell[3], int32_t* launches_per_
  * its buffers, or code on a latency-critical path where cudaMalloc/cudaFree
  * (which can synchronise the device) are not allowed.  This entry point runs
  * the binning and density kernels with all temporaries in one fixed
- * __device__ array of the library (about 4.3 MB, held by every GPU that
+ * __device__ array of the library (about 5.3 MB, held by every GPU that
  * loads the library until the process exits); it calls no allocator.
  * params: box, periodic, rc, rd, precision and rho_self are used.
  * pos: device array of 3n doubles (interleaved xyz); on non-periodic axes

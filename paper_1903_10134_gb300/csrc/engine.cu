@@ -381,11 +381,7 @@ void make_geo_phys(const mdpd_params& p, uint64_t seed, Geo& g, Phys& f)
         g.hi[k] = p.box_lo[k] + p.box[k];
         g.key_lo[k] = f64_key(g.lo[k]);
         g.key_hi[k] = f64_key(g.hi[k]);
-        // below hi by twice the spacing of doubles near the larger face: for
-        // lo <= x < hi_in the difference x - lo rounds to [0, L)
-        const double big = std::max(std::fabs(g.lo[k]), std::fabs(g.hi[k]));
-        const double hi_in = g.hi[k] - 2.0 * (std::nextafter(big, HUGE_VAL) - big);
-        g.key_in[k] = f64_key(hi_in > g.lo[k] ? hi_in : g.lo[k]);
+        g.key_in[k] = f64_key(inside_bound(g.lo[k], g.hi[k]));
         g.h[k] = p.box[k] / m;
         g.inv_h[k] = 1.0 / g.h[k];
         g.ncell *= m;

@@ -5,8 +5,6 @@
 // not depend on the order of the atomics, and a cell's mobile particles come
 // first) and gathers the state into that order with positions re-expressed as
 // offsets from the cell centre.
-#include <cuda_fp16.h>
-
 #include "pair.cuh"
 
 namespace mdpd {
@@ -18,7 +16,7 @@ constexpr int BLOCK = 256;
 // exclusive scan of the cell counts: tiles of SCAN_TILE cells, one block each
 constexpr int SCAN_THREADS = 1024;
 constexpr int SCAN_ITEMS = 4;
-constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
+static_assert(SCAN_TILE == SCAN_THREADS * SCAN_ITEMS, "tile of the scan");
 
 inline unsigned nblocks(int64_t n, int b = BLOCK) { return (unsigned)((n + b - 1) / b); }
 
@@ -218,32 +216,6 @@ __global__ void k_bin_scatter(int n, const uint32_t* __restrict__ cellof,
     src[dst] = (uint32_t)i;
 }
 
-// Insertion sort of each cell's slots by particle id; also clears the cell's
-// count, so the counts are zero whenever a binning starts.
-__global__ void k_cell_sort(int64_t ncell, const uint32_t* __restrict__ start,
-                            uint32_t* __restrict__ key, uint32_t* __restrict__ src,
-                            uint32_t* __restrict__ count)
-{
-    pdl_enter();
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= ncell) return;
-    count[c] = 0u;      // the counts are consumed; leave them zero for the next binning
-    const uint32_t b = start[c], e = start[c + 1];
-    for (uint32_t a = b + 1; a < e; ++a) {
-        const uint32_t k = key[a], s = src[a];
-        uint32_t p = a;
-        while (p > b && key[p - 1] > k) {
-            key[p] = key[p - 1];
-            src[p] = src[p - 1];
-            --p;
-        }
-        key[p] = k;
-        src[p] = s;
-    }
-}
-
-__device__ __forceinline__ uint16_t half_bits(float x) { return __half_as_ushort(__float2half_rn(x)); }
-
 // Order inside each cell by (frozen, particle id), fused with the gather into
 // cell order.  The scatter filled slot a (in atomic order)
 // with key[a] = frozen << 31 | id and
@@ -338,13 +310,7 @@ __global__ void k_rank_gather(int n, int64_t cap, const uint32_t* __restrict__ c
     const float fo[3] = { to_f32(off[0]), to_f32(off[1]), to_f32(off[2]) };
     if constexpr (sizeof(T) == 8)
         fpos[s] = make_float4(fo[0], fo[1], fo[2], __uint_as_float((uint32_t)pt | (uint32_t)q[0] << 3));
-    const Derived<float>& df = ph_g.df;
-    uint16_t* hp = hpos + (size_t)(s >> 2) * 16 + (s & 3u);
-    const float hx = df.h[0];
-    hp[0] = half_bits(fo[1] * df.inv_rc);
-    hp[4] = half_bits(fo[2] * df.inv_rc);
-    hp[8] = half_bits(fmaf((float)(2 * (q[0] & 3) - 3), 0.5f * hx, fo[0]) * df.inv_rc);
-    hp[12] = half_bits(fmaf((float)(2 * ((q[0] + 2) & 3) - 3), 0.5f * hx, fo[0]) * df.inv_rc);
+    store_hpos(hpos, s, fo[0], fo[1], fo[2], q[0], ph_g.df);
     // the random stream is keyed on ids within the replica
     vel4[s] = make4(to_t<T>(vv[0]), to_t<T>(vv[1]), to_t<T>(vv[2]), pack_u32(T(0), pid - id0));
 }
@@ -503,13 +469,6 @@ void launch_bin_scatter(cudaStream_t st, int n, const uint32_t* cellof, const ui
     if (n <= 0) return;
     launch_pdl(k_bin_scatter, dim3(nblocks(n)), dim3(BLOCK), st, n, cellof, slot, start, id, key, src,
                status);
-}
-
-void launch_cell_sort(cudaStream_t st, int64_t ncell, const uint32_t* start, uint32_t* key,
-                      uint32_t* src, uint32_t* count)
-{
-    if (ncell <= 0) return;
-    launch_pdl(k_cell_sort, dim3(nblocks(ncell)), dim3(BLOCK), st, ncell, start, key, src, count);
 }
 
 void launch_rank_gather(cudaStream_t st, int precision, int n, int64_t cap,

@@ -213,9 +213,11 @@ __device__ __forceinline__ void density_home(
     const typename Vec4<T>::type* __restrict__ pos4, const float4* __restrict__ fpos,
     const uint4* __restrict__ hpos, const uint32_t* __restrict__ cell_s,
     const uint32_t* __restrict__ start, T* __restrict__ rho_out, uint32_t* __restrict__ nl,
-    uint32_t* __restrict__ nl_count, unsigned long long* __restrict__ facc, int64_t lcol)
+    uint32_t* __restrict__ nl_count, unsigned long long* __restrict__ facc, int64_t lcol,
+    const uint32_t* __restrict__ src = nullptr, double* __restrict__ out = nullptr)
 {
     static_assert(LPH == 1 || LPH == 4, "lanes per home");
+    constexpr bool LIST = FS != 3;
     const Derived<T>& dc = derived<T>(ph);
     const Derived<float>& df = ph.df;
     const int tid = threadIdx.x;
@@ -270,7 +272,7 @@ __device__ __forceinline__ void density_home(
         }
     };
     const bool mob_true = ((ph.frozen >> type_of(pi.w)) & 1u) == 0u;
-    const bool mobile = ph.list_all || mob_true;
+    const bool mobile = LIST && (ph.list_all || mob_true);
     // wall density of a mobile particle (WANT_PHI): sum over frozen partners
     // within r_c of 15/(2 pi r_c^3) (1 - r/r_c)^2
     const bool want_phi = WANT_PHI && mob_true;
@@ -513,7 +515,7 @@ __device__ __forceinline__ void density_home(
                     if (sub == 0)
                         for (uint32_t k = 0; k < nt; ++k) acc = rho_add(acc, sm.term[k][tid + t]);
                 }
-                for (uint32_t k = 0; k < nhit; ++k)
+                for (uint32_t k = 0; LIST && k < nhit; ++k)
                     if (before + k < (uint32_t)NL_MAX) lp[(int64_t)(before + k) * cap] = sm.hit[k][tid];
                 __syncwarp(group);             // the terms are read before the next home's
                 break;
@@ -526,6 +528,11 @@ __device__ __forceinline__ void density_home(
     }
     }
     if (sub != 0) return;
+    if constexpr (!LIST) {
+        const uint32_t f = src[s], i = f & 0x7fffffffu;
+        if ((int64_t)i < cap) out[i] = f >> 31 ? __longlong_as_double(0x7ff8000000000000ll) : (double)acc;
+        return;
+    }
     rho_out[s] = acc;
     nl_count[s] = cnt;
     if (WANT_PHI) ((T*)ph.phi_out)[s] = phi;
@@ -540,7 +547,8 @@ __device__ __forceinline__ void density_home(
 // addition, so the sum does not depend on the order; k_frozen_rho then forms
 // rho_j = rho_ff + facc * fix_inv and clears facc.  Each FS = 1 block gathers
 // the mobile homes of R * PAIR_BLOCK slots (R = frozen_rounds) and runs them in
-// rounds, so no warp is spent on frozen homes.  FS = 0: every particle is
+// rounds, so no warp is spent on frozen homes.  FS = 3: densities only, to out[src[s]]
+// (NaN where src has its top bit set).  FS = 0: every particle is
 // a home, and partner lists are written for mobile ones (all under list_all).
 template <typename T, bool BATCH, bool WANT_PHI, int FS, int LPH, int R>
 __global__ void __launch_bounds__(PAIR_BLOCK, LPH > 1 ? 4 : sizeof(T) == 4 ? 8 : 5)
@@ -549,7 +557,8 @@ k_density_nl(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
              const uint4* __restrict__ hpos, const uint32_t* __restrict__ cell_s,
              const uint32_t* __restrict__ start, T* __restrict__ rho_out,
              uint32_t* __restrict__ nl, uint32_t* __restrict__ nl_count,
-             unsigned long long* __restrict__ facc)
+             unsigned long long* __restrict__ facc, const uint32_t* __restrict__ src,
+             double* __restrict__ out)
 {
     static_assert(FS == 0 || !BATCH, "the frozen split is for single systems");
     __shared__ DensitySmem<T, LPH> sm;
@@ -616,7 +625,7 @@ k_density_nl(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
     if (k >= count) return;
     density_home<T, WANT_PHI, FS, LPH>(sm, first + k, cap, BATCH ? rp->geo : geo_p,
                                        BATCH ? rp->ph : ph_p, cell0, pos4, fpos, hpos, cell_s, start,
-                                       rho_out, nl, nl_count, facc, (int64_t)(first + k));
+                                       rho_out, nl, nl_count, facc, (int64_t)(first + k), src, out);
 }
 
 }  // namespace
@@ -651,7 +660,7 @@ static void density_t(cudaStream_t st, int n, int64_t cap, const Geo& geo, const
     const int per = fs == 1 ? R * PAIR_BLOCK : PAIR_BLOCK / lph;      // slots of a block
     launch_pdl(k, dim3((n + per - 1) / per), dim3(PAIR_BLOCK), st, n, cap, geo, ph, Batch{},
                (const V*)pos4, (const float4*)fpos, (const uint4*)hpos, cell_s, start, (T*)rho, nl,
-               nl_count, facc);
+               nl_count, facc, (const uint32_t*)nullptr, (double*)nullptr);
     if (fs == 1)
         launch_pdl(k_frozen_rho<T>, dim3(nb), dim3(PAIR_BLOCK), st, n, ph, id_s,
                    (const T*)rho_ff, facc, (T*)rho);
@@ -678,7 +687,25 @@ static void density_batch_t(cudaStream_t st, int64_t cap, const Batch& bt, const
     launch_pdl_smem(k_density_nl<T, true, false, 0, LPH, 1>, dim3(bt.nchunk * LPH), dim3(PAIR_BLOCK),
                     REP_SMEM, st, 0, cap, Geo{}, Phys{}, bt, (const typename Vec4<T>::type*)pos4,
                     (const float4*)fpos, (const uint4*)hpos, cell_s, start, (T*)rho, nl, nl_count,
-                    nullptr);
+                    nullptr, (const uint32_t*)nullptr, (double*)nullptr);
+}
+
+void launch_density_only(cudaStream_t st, int precision, int n, const Geo& geo, const Phys& ph,
+                         const void* pos4, const void* fpos, const uint16_t* hpos,
+                         const uint32_t* cell_s, const uint32_t* start, const uint32_t* src, double* out)
+{
+    if (n <= 0) return;
+    auto go = [&](auto t, auto k, int lph) {
+        using T = decltype(t);
+        const int per = PAIR_BLOCK / lph;
+        launch_pdl(k, dim3((n + per - 1) / per), dim3(PAIR_BLOCK), st, n, (int64_t)n, geo, ph, Batch{},
+                   (const typename Vec4<T>::type*)pos4, (const float4*)fpos, (const uint4*)hpos, cell_s,
+                   start, (T*)nullptr, (uint32_t*)nullptr, (uint32_t*)nullptr,
+                   (unsigned long long*)nullptr, src, out);
+    };
+    if (precision == 0) go(double{}, k_density_nl<double, false, false, 3, 1, 1>, 1);
+    else if (density_lanes(1, n) == 4) go(float{}, k_density_nl<float, false, false, 3, 4, 1>, 4);
+    else go(float{}, k_density_nl<float, false, false, 3, 1, 1>, 1);
 }
 
 void launch_density_nl_batch(cudaStream_t st, int precision, int64_t cap, const Batch& bt,

@@ -42,6 +42,15 @@ struct Geo {
     int64_t ncell;
 };
 
+// Below hi by twice the spacing of doubles near the larger face: for lo <= x below it
+// the difference x - lo rounds to [0, L), so x needs no periodic wrap (Geo::key_in).
+inline double inside_bound(double lo, double hi)
+{
+    const double big = std::fmax(std::fabs(lo), std::fabs(hi));
+    const double in = hi - 2.0 * (std::nextafter(big, HUGE_VAL) - big);
+    return in > lo ? in : lo;
+}
+
 // Constants derived from Phys and Geo in the precision of the pair
 // arithmetic, computed once on the host (FP64 arithmetic runs at a small
 // fraction of the FP32 rate on this part, so kernels must not rederive them
@@ -291,7 +300,7 @@ __device__ __forceinline__ const Rep& block_rep(const Rep* __restrict__ reps, in
 // z x 4, xa x 4, xb x 4 (32 bytes).  y and z are offsets from the cell's centre, xa
 // and xb are measured from the middle of the four cells 4k .. 4k + 3 and 4k - 2 ..
 // 4k + 1 the particle's is one of, all in units of r_c.
-__host__ __device__ inline size_t hpos_words(size_t cap) { return (cap + 7) / 4 * 16; }
+__host__ __device__ constexpr size_t hpos_words(size_t cap) { return (cap + 7) / 4 * 16; }
 
 constexpr int OBS_PARTIALS = 16;   // observable slots per partial (14 used)
 
@@ -304,6 +313,7 @@ void launch_bin_count(cudaStream_t st, int n, int64_t cap, const Geo& geo, const
                       const MaskDev& mk, const Master& m, bool kick, uint32_t* cellof,
                       uint32_t* slot, uint32_t* count, uint32_t* tsum, uint32_t* status);
 int scan_num_blocks(int64_t n);
+constexpr int SCAN_TILE = 4096;        // elements of a scan block
 // Whether the binning of a lattice of n cells forms the scan's tile sums in
 // its count kernel (few tiles) or in a launch of their own.
 bool scan_fused_sums(int64_t n);
@@ -340,10 +350,6 @@ void launch_rank_gather_batch(cudaStream_t st, int precision, int64_t cap, const
 void launch_bin_scatter(cudaStream_t st, int n, const uint32_t* cellof, const uint32_t* slot,
                         const uint32_t* start, const uint32_t* id, uint32_t* key, uint32_t* src,
                         uint32_t* status);
-// Sorts each cell's slots by key and clears count[] for the next binning.
-void launch_cell_sort(cudaStream_t st, int64_t ncell, const uint32_t* start, uint32_t* key,
-                      uint32_t* src, uint32_t* count);
-
 // ---- launchers (pair passes) -----------------------------------------------
 void launch_density(cudaStream_t st, int precision, int n, const Geo& geo, const Phys& ph,
                     const void* pos4, const uint32_t* cell_s, const uint32_t* start, void* rho);
@@ -379,6 +385,11 @@ void launch_density_nl(cudaStream_t st, int precision, int n, int64_t cap, const
                        const uint32_t* cell_s, const uint32_t* start, void* rho, uint32_t* nl, uint32_t* nl_count,
                        int fs = 0, unsigned long long* facc = nullptr,
                        const uint32_t* id_s = nullptr, void* rho_ff = nullptr);
+// Densities of n slots of one mobile type, no lists: out[i] = rho of slot s with
+// i = src[s], or NaN where src[s] has its top bit set.
+void launch_density_only(cudaStream_t st, int precision, int n, const Geo& geo, const Phys& ph,
+                         const void* pos4, const void* fpos, const uint16_t* hpos,
+                         const uint32_t* cell_s, const uint32_t* start, const uint32_t* src, double* out);
 // lpp: lanes per particle (1, 2 or 4).
 void launch_force_nl(cudaStream_t st, int precision, ForceMode mode, int n, int64_t cap,
                      const Geo& geo, const Phys& ph, int lpp, const MaskDev& mk, const void* pos4,

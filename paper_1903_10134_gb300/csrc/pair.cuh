@@ -4,6 +4,8 @@
 // observables.
 #pragma once
 
+#include <cuda_fp16.h>
+
 #include "f64bits.cuh"
 #include "mdpd_internal.cuh"
 #include "philox.cuh"
@@ -416,6 +418,20 @@ __device__ __forceinline__ void finish_obs(const double (&t)[NOBS], uint64_t ste
         for (int k = 0; k < MDPD_NUM_OBS; ++k) obs_sum[k] += o[k];
         *obs_count += 1.0;
     }
+}
+
+// The density filter's FP16 position of slot s (see hpos_words): offsets x, y, z from
+// the centre of its cell, in column q0.
+__device__ __forceinline__ void store_hpos(uint16_t* __restrict__ hpos, uint32_t s, float x, float y,
+                                           float z, int q0, const Derived<float>& df)
+{
+    auto put = [&](int k, float v) {
+        hpos[(size_t)(s >> 2) * 16 + 4 * k + (s & 3u)] = __half_as_ushort(__float2half_rn(v * df.inv_rc));
+    };
+    put(0, y);
+    put(1, z);
+    put(2, fmaf((float)(2 * (q0 & 3) - 3), 0.5f * df.h[0], x));
+    put(3, fmaf((float)(2 * ((q0 + 2) & 3) - 3), 0.5f * df.h[0], x));
 }
 
 // Decompose a cell id into lattice coordinates.
