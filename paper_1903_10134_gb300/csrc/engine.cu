@@ -3,6 +3,7 @@
 // handle's stream (directly or as a captured CUDA graph) and moves data in
 // and out in particle-id order.
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -98,6 +99,7 @@ struct mdpd_handle {
     int force_lpp = 1;               // lanes per particle of the force pass (single system)
     bool walls_set = false;
     std::vector<int32_t> h_type;
+    std::vector<std::array<int64_t, 8>> type_count;   // particles by type (of each replica)
     int64_t steps_host = 0;
 
     // graphs[profiled][mode: 0 fused, 1 last][cur][first half-kick in the binning]
@@ -410,6 +412,19 @@ void make_geo_phys(const mdpd_params& p, uint64_t seed, Geo& g, Phys& f)
     fill_derived(f, g);
 }
 
+// Phys::rho_groups of the system, or of each replica, from its mobile particles (once
+// the types are known).
+void set_rho_groups(mdpd_handle* h)
+{
+    for (size_t r = 0; r < h->type_count.size(); ++r) {
+        Phys& ph = h->nrep ? h->reps[r].ph : h->ph;
+        int64_t mobile = 0;
+        for (int t = 0; t < 8; ++t)
+            if (!((ph.frozen >> t) & 1u)) mobile += h->type_count[r][t];
+        ph.rho_groups = density_groups(mobile) ? 1 : 0;
+    }
+}
+
 void setup_geo_phys(mdpd_handle* h)
 {
     const int list_all = h->ph.list_all;
@@ -418,6 +433,7 @@ void setup_geo_phys(mdpd_handle* h)
     make_geo_phys(h->p, h->seed, h->geo, h->ph);
     h->ph.list_all = list_all;
     h->ph.dbg_status = h->status;
+    set_rho_groups(h);
 }
 
 int status_to_code(uint32_t st)
@@ -822,6 +838,10 @@ int init_handle(mdpd_handle* h, const double* pos, const double* vel, const int3
                     return bail(MDPD_ERR_INVALID_ARG);
                 }
     }
+    h->type_count.assign(bounds.size() - 1, {});
+    for (size_t r = 0; r + 1 < bounds.size(); ++r)
+        for (int64_t i = bounds[r]; i < bounds[r + 1]; ++i) ++h->type_count[r][h->h_type[i]];
+    set_rho_groups(h);
     if ((rc = alloc_particles(h, n))) return bail(rc);
     const int64_t nb = scan_num_blocks(h->geo.ncell);
     if ((rc = dalloc(h, &h->count, (size_t)h->geo.ncell * sizeof(uint32_t))) ||
@@ -1103,6 +1123,7 @@ int mdpd_batch_set_params(mdpd_handle* h, const mdpd_params* params)
         philox_round_keys(k0, k1, R.ph.rk);
         h->rep_p[r] = params[r];
     }
+    set_rho_groups(h);
     // the records live in device memory: captured graphs stay valid
     h->win_valid = false;
     return upload_reps(h);
@@ -1224,7 +1245,9 @@ int mdpd_set_walls(mdpd_handle* h, const uint8_t* solid, int32_t nx, int32_t ny,
         return h->fail(MDPD_ERR_CUDA, "wall emission failed");
     }
     h->n = n_new;
+    h->type_count[0][wall_type] += n_new - (int64_t)h->h_type.size();
     h->h_type.resize((size_t)n_new, wall_type);
+    set_rho_groups(h);
     dfree(h->mask_bits);
     h->mask_bits = bits;
     h->mk.bits = bits;

@@ -136,14 +136,18 @@ k_frozen_part(int n, int64_t cap, Geo geo, Phys ph, const typename Vec4<T>::type
 // (empty ones skipped) take the places of those runs.  A home with more masks than
 // that (runs longer than 32 candidates) works them off and goes on.
 //
-// LPH lanes share a home in small systems (density_lanes), where one lane's chain of
-// 5,000 instructions is the pass's time: the lanes take the rows 0 - 3, 4 (its own, with
-// ten of the 25 hits), 5 - 6 and 7 - 8, and their hits and density terms wait in
-// shared memory.  The list
-// is then the lanes' hits one after another and one lane adds the terms in that
-// order, so lists and sums are those of one lane.  A home whose lanes' hits do not
-// fit is done again by one lane after the other.
-constexpr int DN_HITS = 24;        // hits and terms kept per lane (LPH > 1)
+// The rows are taken in the order of dn_row: the home's own, with ten of the 25 hits, then
+// three, three and two of the others.  LPH = 4 lanes share a home in systems of few
+// particles (density_groups), where one lane's chain of 5,000 instructions is the pass's
+// time: each takes one of these groups.  The home's hits wait in shared memory, each
+// lane's behind the filter's count of those before it; the list is the lanes' hits one
+// after another and the density the sum of theirs in that order.  A home whose hits do not
+// fit counts them first and finds them again for the list.  In a batch a replica's home
+// may have one lane where its system alone has four: the lane then sums the groups apart
+// as well (ph.rho_groups, fold), so that the replica stays that system to the bit.
+__device__ constexpr int dn_row(int k) { return (int)(0x867523104ull >> 4 * k & 15u); }
+constexpr uint32_t DN_GROUP = 0x3b865u;       // group of a row, two bits each
+constexpr int DN_POOL = 57;        // a home's hits (LPH > 1); odd, for the banks
 // r^2 < FILT passes (1 + 9 * 2^-10, exact in FP16).  With u = 2^-10 an |x| < 4 is off by
 // u at most, home and candidate; |y|, |z| < 1 of a candidate by u / 4, < 3 of a home
 // by u; a difference near 1 by u / 2 more.  That is 2.5 u in x and 1.75 u in y and z,
@@ -153,18 +157,17 @@ constexpr float FILT = 1.0f + 9.0f / 1024.0f;
 
 template <typename T, int LPH>
 struct DensitySmem {
-    static constexpr int RUNS = LPH == 1 ? 18 : 8;     // two for each of a lane's rows
+    static constexpr int RUNS = LPH == 1 ? 18 : 6;     // two for each of a lane's rows
     // FP64: candidates near r_d kept before they are evaluated
     static constexpr int NEAR = sizeof(T) == 4 ? 1 : 32;
-    // run: length, first slot | row << 27 | across a face in x << 31
-    // mask: candidates from the top bit, first slot | row << 27 | across << 31
+    // run: length, first slot | across a face in x << 27 | row << 28
+    // mask: candidates from the top bit, first slot | across << 27 | row << 28
     uint32_t a[RUNS][PAIR_BLOCK];
     uint32_t b[RUNS][PAIR_BLOCK];
     typename Vec4<T>::type shift[27];          // image shift of a neighbour-cell code
     float4 fshift[sizeof(T) == 8 ? 27 : 1];    // the same in FP32
-    uint32_t near[NEAR][PAIR_BLOCK];
-    uint32_t hit[LPH == 1 ? 1 : DN_HITS][PAIR_BLOCK];
-    T term[LPH == 1 ? 1 : DN_HITS][PAIR_BLOCK];
+    uint32_t near[NEAR][sizeof(T) == 4 ? 1 : PAIR_BLOCK];
+    uint32_t hit[LPH == 1 ? 1 : PAIR_BLOCK / LPH][DN_POOL];
 };
 
 // Density terms and sums with each operation rounded, so that the two ways of
@@ -207,7 +210,7 @@ __device__ __forceinline__ void fill_shift(DensitySmem<T, LPH>& sm, const Phys& 
 
 // The density and partner list of the home in slot s; column lcol of the list.
 // With LPH > 1 the LPH lanes of a group call it together.
-template <typename T, bool WANT_PHI, int FS, int LPH>
+template <typename T, bool WANT_PHI, int FS, int LPH, bool FOLD>
 __device__ __forceinline__ void density_home(
     DensitySmem<T, LPH>& sm, int s, int64_t cap, const Geo& geo, const Phys& ph, int64_t cell0,
     const typename Vec4<T>::type* __restrict__ pos4, const float4* __restrict__ fpos,
@@ -231,20 +234,21 @@ __device__ __forceinline__ void density_home(
     // the part across the upper one last
     const bool lo_x = geo.periodic[0] && q0 == 0, hi_x = geo.periodic[0] && q0 == geo.nc[0] - 1;
     const int xb0 = max(q0 - 1, 0), xe0 = min(q0 + 1, geo.nc[0] - 1) + 1;
-    constexpr int ROWS = LPH == 1 ? 9 : 4;
-    const int row0 = LPH == 1 ? 0 : (0x97540 >> 4 * sub) & 15, row1 = LPH == 1 ? 9 : (0x9754 >> 4 * sub) & 15;
+    constexpr int ROWS = LPH == 1 ? 9 : 3;
+    const int k0 = LPH == 1 ? 0 : (0x7410 >> 4 * sub) & 15, kend = LPH == 1 ? 9 : (0x9741 >> 4 * sub) & 15;
     int nrun = 0;
     auto build_runs = [&]() {
         uint32_t b[ROWS], e[ROWS];
-        auto row_start = [&](int r) -> const uint32_t* {
-            const int z = neighbour_index(q2, r / 3 - 1, geo.nc[2], geo.periodic[2]);
-            const int y = neighbour_index(q1, r % 3 - 1, geo.nc[1], geo.periodic[1]);
-            return r < row1 && z >= 0 && y >= 0 ? start + cell0 + geo.nc[0] * (y + geo.nc[1] * z)
+        auto row_start = [&](int k) -> const uint32_t* {
+            const int r = dn_row(k), oz = r * 11 >> 5;
+            const int z = neighbour_index(q2, oz - 1, geo.nc[2], geo.periodic[2]);
+            const int y = neighbour_index(q1, r - 3 * oz - 1, geo.nc[1], geo.periodic[1]);
+            return k < kend && z >= 0 && y >= 0 ? start + cell0 + geo.nc[0] * (y + geo.nc[1] * z)
                                                 : nullptr;
         };
 #pragma unroll
         for (int k = 0; k < ROWS; ++k) {
-            const uint32_t* st = row_start(row0 + k);
+            const uint32_t* st = row_start(k0 + k);
             b[k] = st ? st[xb0] : 0u;
             e[k] = st ? st[xe0] : 0u;
         }
@@ -258,16 +262,16 @@ __device__ __forceinline__ void density_home(
         };
 #pragma unroll
         for (int k = 0; k < ROWS; ++k) {
-            const uint32_t r = (uint32_t)(row0 + k);
+            const uint32_t r = (uint32_t)dn_row(k0 + k);
             if (lo_x || hi_x) {
-                const uint32_t* st = row_start((int)r);
+                const uint32_t* st = row_start(k0 + k);
                 if (!st) continue;
                 const int x = lo_x ? geo.nc[0] - 1 : 0;
-                if (hi_x) put(b[k], e[k], r);
-                put(st[x], st[x + 1], r | 16u);
-                if (lo_x) put(b[k], e[k], r);
+                if (hi_x) put(b[k], e[k], r << 1);
+                put(st[x], st[x + 1], r << 1 | 1u);
+                if (lo_x) put(b[k], e[k], r << 1);
             } else {
-                put(b[k], e[k], r);
+                put(b[k], e[k], r << 1);
             }
         }
     };
@@ -277,6 +281,18 @@ __device__ __forceinline__ void density_home(
     // within r_c of 15/(2 pi r_c^3) (1 - r/r_c)^2
     const bool want_phi = WANT_PHI && mob_true;
     T acc = ph.rho_self ? dc.cw_rho : T(0), phi = T(0);
+    // part: the sum of the current group of rows, which fold adds to acc
+    T part = acc;
+    acc = T(0);
+    if (LPH > 1 && sub != 0) part = T(0);
+    uint32_t group_now = 0;
+    auto fold = [&](uint32_t jr) {
+        const uint32_t g = (DN_GROUP >> 2 * (jr >> 28)) & 3u;
+        if (g == group_now) return;
+        acc = rho_add(acc, part);
+        part = T(0);
+        group_now = g;
+    };
     uint32_t cnt = 0;
     uint32_t* lp = nl + lcol;                   // next list entry: nl[cnt * cap + lcol]
     // cell column of a candidate across a periodic face, from the home's
@@ -295,29 +311,35 @@ __device__ __forceinline__ void density_home(
     __half2 hx = hx0, hy = hx0, hz = hx0;
     bool xb = win_b;
 
-    // pass 0: every lane its rows (LPH > 1: hits and terms kept); passes 1 .. LPH, if
-    // a lane's did not fit: the lanes in turn, straight to the list and the sum
-    uint32_t nhit = 0, nterm = 0;
-    for (int pass = 0; pass <= (LPH == 1 ? 0 : LPH); ++pass) {
-    const bool keep = LPH > 1 && pass == 0;
-    if (LPH == 1 || pass == 0 || sub == pass - 1) {
+    // pass 0: every lane its rows (LPH > 1: hits kept, or counted if they do not fit);
+    // pass 1, if they did not: once more for the list
+    uint32_t nhit = 0, pool = 0;
+    bool fits = true;
+    for (int pass = 0; pass < (LPH == 1 ? 1 : 2); ++pass) {
     build_runs();
+    // place of mask k: the runs' done ones, before them (LPH > 1) the never used ones
+    auto place = [&](int k) {
+        if (LPH == 1) return k;
+        const int q = nrun + k;
+        return q >= DensitySmem<T, LPH>::RUNS ? q - DensitySmem<T, LPH>::RUNS : q;
+    };
     int run = 0;
     uint32_t len = 0, rb = 0;
-    while (run < nrun || len) {
+    for (bool first = LPH > 1 && pass == 0; first || run < nrun || len; first = false) {
         int nw = 0;
+        uint32_t npass = 0;
         while (run < nrun || len) {
             uint32_t lead = 0;
             if (len == 0) {
                 len = sm.a[run][tid];
                 rb = sm.b[run][tid];
                 ++run;
-                const int r = (int)((rb >> 27) & 15u), rz = (r * 11) >> 5, ry = r - 3 * rz;
+                const int r = (int)(rb >> 28), rz = (r * 11) >> 5, ry = r - 3 * rz;
                 hy = __float2half2_rn(fmaf(small_float((uint32_t)ry) - 1.0f, -hn1, oy1));
                 hz = __float2half2_rn(fmaf(small_float((uint32_t)rz) - 1.0f, -hn2, oz1));
                 hx = hx0;
                 xb = win_b;
-                if ((int)rb < 0) {
+                if (rb & 1u << 27) {
                     // across a periodic face: one cell, met from the column beside it
                     hx = q0 == 0 ? x_in_window(geo.nc[0] - 1, 1) : x_in_window(0, -1);
                     xb = false;
@@ -347,54 +369,56 @@ __device__ __forceinline__ void density_home(
             const uint32_t self = (uint32_t)s - (rb & 0x07ffffffu);
             if (self < 32u) m &= ~(0x80000000u >> self);
             if (m) {
-                sm.a[nw][tid] = m;
-                sm.b[nw][tid] = rb;
+                sm.a[place(nw)][tid] = m;
+                sm.b[place(nw)][tid] = rb;
                 ++nw;
+                if (LPH > 1) npass += (uint32_t)__popc(m);
             }
             rb += k1;
             len -= k1;
-            if (nw == run && len) break;       // no place free until masks are worked off
+            // no place free until masks are worked off
+            if (nw == run + (LPH > 1 ? DensitySmem<T, LPH>::RUNS - nrun : 0) && len) break;
+        }
+        if (LPH > 1 && first) {
+            uint32_t all = 0;
+#pragma unroll
+            for (int t = 0; t < LPH; ++t) {
+                const uint32_t nt = __shfl_sync(group, npass, t, LPH);
+                pool += t < sub ? nt : 0u;
+                all += nt;
+            }
+            fits = __all_sync(group, all <= (uint32_t)DN_POOL && run == nrun && len == 0u);
         }
         if (nw == 0) break;
 
         // the set bits, one ahead of the one worked on
         int w = 0;
-        uint32_t m = sm.a[0][tid], base = sm.b[0][tid];
+        uint32_t m = sm.a[place(0)][tid], base = sm.b[place(0)][tid];
         uint32_t j1 = 0;
         auto next = [&]() {
             const int b = __clz((int)m);
             j1 = base + (uint32_t)b;           // row and face bits above the slot
             m ^= 0x80000000u >> b;
             if (m == 0u && ++w < nw) {
-                m = sm.a[w][tid];
-                base = sm.b[w][tid];
+                m = sm.a[place(w)][tid];
+                base = sm.b[place(w)][tid];
             }
         };
         // neighbour-cell code of a candidate in cell column qj, jr as from next()
         auto code_of = [&](uint32_t qj, uint32_t jr) {
-            const int ox = (int)qj - q0 + ((int)jr < 0 ? across : 0);
-            return 3 * (int)((jr >> 27) & 15u) + ox + 1;
+            const int ox = (int)qj - q0 + (jr & 1u << 27 ? across : 0);
+            return 3 * (int)(jr >> 28) + ox + 1;
         };
         auto append = [&](uint32_t j, int code) {
             const uint32_t entry = j << 5 | (uint32_t)code;   // (bits above the slot shift out)
-            if (LPH > 1 && keep) {
-                if (nhit < (uint32_t)DN_HITS) sm.hit[nhit][tid] = entry;
+            if (LPH > 1 && pass == 0) {
+                if (fits) sm.hit[tid / LPH][pool + nhit] = entry;
                 ++nhit;
                 return;
             }
             if (cnt < (uint32_t)NL_MAX) *lp = entry;
             lp += cap;
             ++cnt;
-        };
-        auto add = [&](T term) {
-            if (LPH > 1 && keep) {
-                if (term > T(0)) {
-                    if (nterm < (uint32_t)DN_HITS) sm.term[nterm][tid] = term;
-                    ++nterm;
-                }
-                return;
-            }
-            acc = rho_add(acc, term);
         };
         next();
         if constexpr (sizeof(T) == 4) {
@@ -416,7 +440,10 @@ __device__ __forceinline__ void density_home(
                 if (r2 < dc.rc2) {
                     const float wr = max(1.0f - sqrt_fast(r2) * dc.inv_rd, 0.0f);
                     const float term = rho_term(dc.cw_rho, wr);  // r = 0 gives w(0)
-                    add(term);
+                    if (pass == 0) {
+                        if (FOLD && ph.rho_groups) fold(jr);
+                        part = rho_add(part, term);
+                    }
                     const bool fz = (FS == 1 || WANT_PHI) && ((ph.frozen >> (bits & 7u)) & 1u);
                     if (FS == 1 && fz && term > 0.0f && pass == 0)
                         atomicAdd(facc + (jr & 0x07ffffffu), to_fixed(term * dc.fix_scale));
@@ -449,8 +476,8 @@ __device__ __forceinline__ void density_home(
                 if (r2 < dc.rc2) {
                     const T wr = max(T(1) - sqrt_fast(r2) * dc.inv_rd, T(0));
                     const T term = rho_term(dc.cw_rho, wr);      // r = 0 gives w(0)
-                    add(term);
-                    const bool fz = (FS == 1 || WANT_PHI) && pass == 0 &&
+                    part = rho_add(part, term);
+                    const bool fz = (FS == 1 || WANT_PHI) &&
                                     ((ph.frozen >> type_of(pos4[j].w)) & 1u);
                     if (FS == 1 && fz && term > T(0))
                         atomicAdd(facc + j, to_fixed(term * dc.fix_scale));
@@ -495,37 +522,34 @@ __device__ __forceinline__ void density_home(
             evaluate_near();
         }
     }
+    if constexpr (LPH > 1) {
+        if (pass == 1) break;
+        uint32_t all = 0;
+#pragma unroll
+        for (int t = 0; t < LPH; ++t) {
+            const uint32_t ht = __shfl_sync(group, nhit, t, LPH);
+            acc = rho_add(acc, __shfl_sync(group, part, t, LPH));
+            cnt += t < sub ? ht : 0u;
+            all += ht;
+        }
+        // wall density: the lanes' sums in a fixed order
+        if (WANT_PHI)
+#pragma unroll
+            for (int o = 1; o < LPH; o <<= 1) phi += __shfl_xor_sync(group, phi, o);
+        if (LIST && fits)
+            for (uint32_t k = 0; k < nhit; ++k)
+                if (cnt + k < (uint32_t)NL_MAX)
+                    lp[(int64_t)(cnt + k) * cap] = sm.hit[tid / LPH][pool + k];
+        lp += (int64_t)cnt * cap;
+        pool = all;                            // the home's hits
+        if (!LIST || fits || all == 0u) break;
+    }
     }
     if constexpr (LPH > 1) {
-        __syncwarp(group);
-        if (pass == 0) {
-            const bool fits = nhit <= (uint32_t)DN_HITS && nterm <= (uint32_t)DN_HITS;
-            // wall density: the lanes' sums in a fixed order
-            if (WANT_PHI)
-#pragma unroll
-                for (int o = 1; o < LPH; o <<= 1) phi += __shfl_xor_sync(group, phi, o);
-            if (__all_sync(group, fits)) {
-                uint32_t before = 0;
-#pragma unroll
-                for (int t = 0; t < LPH; ++t) {
-                    const uint32_t ht = __shfl_sync(group, nhit, t, LPH);
-                    const uint32_t nt = __shfl_sync(group, nterm, t, LPH);
-                    before += t < sub ? ht : 0u;
-                    cnt += ht;
-                    if (sub == 0)
-                        for (uint32_t k = 0; k < nt; ++k) acc = rho_add(acc, sm.term[k][tid + t]);
-                }
-                for (uint32_t k = 0; LIST && k < nhit; ++k)
-                    if (before + k < (uint32_t)NL_MAX) lp[(int64_t)(before + k) * cap] = sm.hit[k][tid];
-                __syncwarp(group);             // the terms are read before the next home's
-                break;
-            }
-        } else {
-            acc = __shfl_sync(group, acc, pass - 1, LPH);
-            cnt = __shfl_sync(group, cnt, pass - 1, LPH);
-            lp = nl + lcol + (int64_t)cnt * cap;
-        }
-    }
+        cnt = pool;
+        __syncwarp(group);                     // the pool is read before the next home's
+    } else {
+        acc = rho_add(acc, part);
     }
     if (sub != 0) return;
     if constexpr (!LIST) {
@@ -550,8 +574,14 @@ __device__ __forceinline__ void density_home(
 // rounds, so no warp is spent on frozen homes.  FS = 3: densities only, to out[src[s]]
 // (NaN where src has its top bit set).  FS = 0: every particle is
 // a home, and partner lists are written for mobile ones (all under list_all).
+//
+// Bound by issue (82 % of the cycles, L1 data path 70 %): per 32 homes 376 instructions
+// for the runs, 2,228 in the filter, 2,421 for the hits.  Density pass in FP32 before
+// (each candidate in full by one thread, or a warp per cell) and with the filter, us:
+// slab of 820,000 219 / 141, rock of 256^3 voxels (frozen split) 776 / 480, batch of 256
+// liquids (2.8 million) 710 / 476; small systems at density_groups.
 template <typename T, bool BATCH, bool WANT_PHI, int FS, int LPH, int R>
-__global__ void __launch_bounds__(PAIR_BLOCK, LPH > 1 ? 4 : sizeof(T) == 4 ? 8 : 5)
+__global__ void __launch_bounds__(PAIR_BLOCK, sizeof(T) == 4 ? 8 : 5)
 k_density_nl(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
              const typename Vec4<T>::type* __restrict__ pos4, const float4* __restrict__ fpos,
              const uint4* __restrict__ hpos, const uint32_t* __restrict__ cell_s,
@@ -563,14 +593,16 @@ k_density_nl(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
     static_assert(FS == 0 || !BATCH, "the frozen split is for single systems");
     __shared__ DensitySmem<T, LPH> sm;
     constexpr int HOMES = PAIR_BLOCK / LPH;    // homes of a round
+    constexpr bool FOLD = BATCH && LPH == 1 && sizeof(T) == 4;
     pdl_enter();
     if constexpr (FS == 1) {
-        // the mobile homes of the block's R * PAIR_BLOCK slots, in slot order
+        // the mobile homes of R * PAIR_BLOCK slots, in slot order (LPH blocks share
+        // them: each takes HOMES of every PAIR_BLOCK)
         __shared__ int act[R * PAIR_BLOCK];
         __shared__ uint32_t wcnt[R][PAIR_BLOCK / 32];
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
         const unsigned lt = (1u << lane) - 1u;
-        const int64_t base = (int64_t)blockIdx.x * (R * PAIR_BLOCK);
+        const int64_t base = (int64_t)(blockIdx.x / LPH) * (R * PAIR_BLOCK);
         fill_shift(sm, ph_p);
         unsigned bm[R];
 #pragma unroll
@@ -598,8 +630,8 @@ k_density_nl(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
         // slot plus the home's place among its mobile homes, which the force
         // pass's rounds blocks form the same way (consecutive columns for a
         // warp's homes: coalesced list stores and loads)
-        for (uint32_t q = threadIdx.x / LPH; q < nmob; q += HOMES)
-            density_home<T, WANT_PHI, FS, LPH>(sm, act[q], cap, geo_p, ph_p, 0, pos4, fpos, hpos,
+        for (uint32_t q = blockIdx.x % LPH * HOMES + threadIdx.x / LPH; q < nmob; q += PAIR_BLOCK)
+            density_home<T, WANT_PHI, FS, LPH, false>(sm, act[q], cap, geo_p, ph_p, 0, pos4, fpos, hpos,
                                                cell_s, start, rho_out, nl, nl_count, facc,
                                                ph_p.list_compact ? base + q : (int64_t)act[q]);
         return;
@@ -623,18 +655,12 @@ k_density_nl(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
     __syncthreads();
     const int k = (int)threadIdx.x / LPH;
     if (k >= count) return;
-    density_home<T, WANT_PHI, FS, LPH>(sm, first + k, cap, BATCH ? rp->geo : geo_p,
+    density_home<T, WANT_PHI, FS, LPH, FOLD>(sm, first + k, cap, BATCH ? rp->geo : geo_p,
                                        BATCH ? rp->ph : ph_p, cell0, pos4, fpos, hpos, cell_s, start,
                                        rho_out, nl, nl_count, facc, (int64_t)(first + k), src, out);
 }
 
 }  // namespace
-
-// Lanes that share a home in a pass over n slots in which every particle is a home.
-// Measured, density pass in FP32 with one lane and with four: 1,000 particles 25 and
-// 18 us, 4,000 28 and 19, 12,000 27 and 20, 20,000 27 and 29, 40,000 28 and 41.  FP64
-// (the terms of the middle row, half of them, are one lane's) 53 and 63 us at 1,000.
-static int density_lanes(int precision, int64_t n) { return precision == 1 && n <= 16000 ? 4 : 1; }
 
 template <typename T, int R>
 static void density_t(cudaStream_t st, int n, int64_t cap, const Geo& geo, const Phys& ph,
@@ -651,13 +677,14 @@ static void density_t(cudaStream_t st, int n, int64_t cap, const Geo& geo, const
         return;
     }
     const bool phi = ph.phi_out != nullptr;
-    const int lph = fs == 1 ? 1 : density_lanes(sizeof(T) == 8 ? 0 : 1, n);
+    const int lph = sizeof(T) == 4 && R == 1 && ph.rho_groups ? 4 : 1;
     auto k = fs == 1 ? (phi ? k_density_nl<T, false, true, 1, 1, R> : k_density_nl<T, false, false, 1, 1, R>)
                      : (phi ? k_density_nl<T, false, true, 0, 1, 1> : k_density_nl<T, false, false, 0, 1, 1>);
-    if constexpr (sizeof(T) == 4)
+    if constexpr (sizeof(T) == 4 && R == 1)
         if (lph == 4)
-            k = phi ? k_density_nl<T, false, true, 0, 4, 1> : k_density_nl<T, false, false, 0, 4, 1>;
-    const int per = fs == 1 ? R * PAIR_BLOCK : PAIR_BLOCK / lph;      // slots of a block
+            k = fs == 1 ? (phi ? k_density_nl<T, false, true, 1, 4, R> : k_density_nl<T, false, false, 1, 4, R>)
+                        : (phi ? k_density_nl<T, false, true, 0, 4, 1> : k_density_nl<T, false, false, 0, 4, 1>);
+    const int per = (fs == 1 ? R * PAIR_BLOCK : PAIR_BLOCK) / lph;     // slots of a block
     launch_pdl(k, dim3((n + per - 1) / per), dim3(PAIR_BLOCK), st, n, cap, geo, ph, Batch{},
                (const V*)pos4, (const float4*)fpos, (const uint4*)hpos, cell_s, start, (T*)rho, nl,
                nl_count, facc, (const uint32_t*)nullptr, (double*)nullptr);
@@ -704,7 +731,7 @@ void launch_density_only(cudaStream_t st, int precision, int n, const Geo& geo, 
                    (unsigned long long*)nullptr, src, out);
     };
     if (precision == 0) go(double{}, k_density_nl<double, false, false, 3, 1, 1>, 1);
-    else if (density_lanes(1, n) == 4) go(float{}, k_density_nl<float, false, false, 3, 4, 1>, 4);
+    else if (density_groups(n)) go(float{}, k_density_nl<float, false, false, 3, 4, 1>, 4);
     else go(float{}, k_density_nl<float, false, false, 3, 1, 1>, 1);
 }
 
@@ -715,8 +742,8 @@ void launch_density_nl_batch(cudaStream_t st, int precision, int64_t cap, const 
 {
     if (bt.nchunk <= 0) return;
     auto f = precision == 0 ? density_batch_t<double, 1>
-             : density_lanes(precision, (int64_t)bt.nchunk * PAIR_BLOCK) == 4 ? density_batch_t<float, 4>
-                                                                             : density_batch_t<float, 1>;
+             : density_groups((int64_t)bt.nchunk * PAIR_BLOCK) ? density_batch_t<float, 4>
+                                                               : density_batch_t<float, 1>;
     f(st, cap, bt, pos4, fpos, hpos, cell_s, start, rho, nl, nl_count);
 }
 

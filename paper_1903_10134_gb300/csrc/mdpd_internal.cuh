@@ -51,6 +51,17 @@ inline double inside_bound(double lo, double hi)
     return in > lo ? in : lo;
 }
 
+// Whether the FP32 density pass of a system with this many mobile particles gives each
+// home four lanes (k_density.cu): as long as they fit the chip at once, 152 SMs x 8
+// blocks x 32 homes, for then a home's chain of instructions is the pass's time.
+// Density pass with one lane a home, with four, and that of a warp per cell which these
+// replaced, us: 1,000 particles 25 / 16 / 20, 8,000 27 / 17 / 20, 20,000 27 / 19 / 22,
+// 30,000 27 / 22 / 24, 38,000 28 / 25 / 26, 40,000 28 / 29 / 26, 80,000 33 / 46 / 41; a
+// slit of 38,000 with a collapsed liquid, whose dense homes are the pass, 58 / 39 / 33.
+// (FP64: the terms of the middle row, half of them, are one lane's, and four lanes take
+// longer at every size.)
+inline bool density_groups(int64_t homes) { return homes <= 152 * 8 * 32; }
+
 // Constants derived from Phys and Geo in the precision of the pair
 // arithmetic, computed once on the host (FP64 arithmetic runs at a small
 // fraction of the FP32 rate on this part, so kernels must not rederive them
@@ -85,6 +96,7 @@ struct Phys {
     int list_all;                 // 1: the density pass lists partners of frozen particles too
     int list_compact;             // 1: list column = block base + compacted mobile position
                                   //    (frozen-split density pass and rounds force pass)
+    int rho_groups;               // 1: density sums in four groups of rows (density_groups)
     int prec32;                   // 1: FP32 pair arithmetic (kick increments formed in FP32)
     uint32_t fast_cell;           // bit k: axis k may take cell indices in FP32 (see k_bin_count)
     void* phi_out;                // wall density output (cell order, FP32/FP64), or nullptr
