@@ -50,3 +50,24 @@ def test_frozen_split_with_shared_homes(box):
         assert np.abs(rho - o.rho).max() <= RHO_TOL[1] * o.rho.max()
         phi, ref = s.wall_density(), o.wall_density()
         assert np.abs(phi - ref).max() <= 2e-5 * (1.0 + ref.max())
+
+
+@pytest.mark.parametrize("n, box, frozen", [(39100, (19.0, 18.2, 18.9), (1,)),
+                                            (39100, (12.1, 11.0, 13.2), (1, 2))])
+def test_frozen_split_above_the_size_of_shared_homes(n, box, frozen):
+    """More slots than fit the chip at once, but few enough mobile ones: the split with
+    four lanes a home, at a usual density and at one with more hits than they keep."""
+    from paper_1903_10134_gb300 import mdpd as M
+    w = I.tiny(n, box, 82, periodic=(1, 0, 1), ntypes=3, precision=1, frozen_types=frozen)
+    w.vel[np.isin(w.type, frozen)] = 0.0
+    o = O.Oracle(w.params.copy(precision=0), w.pos, w.vel, w.type, w.seed, use_cells=1)
+    with M.System(w.params, w.pos, w.vel, w.type, w.seed) as s, \
+            M.System(w.params, w.pos, w.vel, w.type, w.seed) as d:
+        s.set_option(M.OPT_WALL_DENSITY, 1)
+        d.set_option(M.OPT_KERNELS, M.KERNELS_SCAN)
+        _, rho = s.forces()
+        d.forces()
+        assert s.pair_count() == d.pair_count()
+        assert np.abs(rho - o.rho).max() <= RHO_TOL[1] * o.rho.max()
+        phi, ref = s.wall_density(), o.wall_density()
+        assert np.abs(phi - ref).max() <= 2e-5 * (1.0 + ref.max())
