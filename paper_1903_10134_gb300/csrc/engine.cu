@@ -418,10 +418,14 @@ void set_rho_groups(mdpd_handle* h)
 {
     for (size_t r = 0; r < h->type_count.size(); ++r) {
         Phys& ph = h->nrep ? h->reps[r].ph : h->ph;
-        int64_t mobile = 0;
-        for (int t = 0; t < 8; ++t)
+        int64_t mobile = 0, all = 0;
+        for (int t = 0; t < 8; ++t) {
+            all += h->type_count[r][t];
             if (!((ph.frozen >> t) & 1u)) mobile += h->type_count[r][t];
-        ph.rho_groups = density_groups(mobile) ? 1 : 0;
+        }
+        // (blocks that work in rounds have one lane for a home)
+        const bool rounds = ph.frozen && frozen_rounds(all) > 1;
+        ph.rho_groups = density_groups(mobile) && !rounds ? 1 : 0;
     }
 }
 

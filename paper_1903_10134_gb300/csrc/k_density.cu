@@ -136,18 +136,19 @@ k_frozen_part(int n, int64_t cap, Geo geo, Phys ph, const typename Vec4<T>::type
 // (empty ones skipped) take the places of those runs.  A home with more masks than
 // that (runs longer than 32 candidates) works them off and goes on.
 //
-// The rows are taken in the order of dn_row: the home's own, with ten of the 25 hits, then
-// three, three and two of the others.  LPH = 4 lanes share a home in systems of few
-// particles (density_groups), where one lane's chain of 5,000 instructions is the pass's
-// time: each takes one of these groups.  The home's hits wait in shared memory, each
-// lane's behind the filter's count of those before it; the list is the lanes' hits one
-// after another and the density the sum of theirs in that order.  A home whose hits do not
-// fit counts them first and finds them again for the list.  In a batch a replica's home
-// may have one lane where its system alone has four: the lane then sums the groups apart
-// as well (ph.rho_groups, fold), so that the replica stays that system to the bit.
-__device__ constexpr int dn_row(int k) { return (int)(0x867523104ull >> 4 * k & 15u); }
-constexpr uint32_t DN_GROUP = 0x3b865u;       // group of a row, two bits each
-constexpr int DN_POOL = 57;        // a home's hits (LPH > 1); odd, for the banks
+// The rows are taken in the order of dn_row, in four groups: the home's own, with ten of
+// the 25 hits, then three, two and three of the others, with two, six and seven.  In
+// systems of few particles (density_groups), where one lane's chain of 5,000 instructions
+// is the pass's time, LPH = 4 lanes share a home and take one group each.  The first
+// writes its hits to the list; those of the others wait in shared memory, each lane's
+// behind the filter's count of those before it, and follow it; the density is the sum of
+// the groups' in their order.  A home whose hits do not fit counts them first and finds
+// them again for the list.  In a batch a replica's home may have one lane where its
+// system alone has four: the lane then sums the groups apart as well (ph.rho_groups,
+// fold), so that the replica stays that system to the bit.
+__device__ constexpr int dn_row(int k) { return (int)(0x75318624ull >> 4 * k & 15u); }
+constexpr uint32_t DN_GROUP = 0x1dc9bu;       // group of a row, two bits each
+constexpr int DN_POOL = 45;        // hits kept for a home (LPH > 1); odd, for the banks
 // r^2 < FILT passes (1 + 9 * 2^-10, exact in FP16).  With u = 2^-10 an |x| < 4 is off by
 // u at most, home and candidate; |y|, |z| < 1 of a candidate by u / 4, < 3 of a home
 // by u; a difference near 1 by u / 2 more.  That is 2.5 u in x and 1.75 u in y and z,
@@ -157,7 +158,8 @@ constexpr float FILT = 1.0f + 9.0f / 1024.0f;
 
 template <typename T, int LPH>
 struct DensitySmem {
-    static constexpr int RUNS = LPH == 1 ? 18 : 6;     // two for each of a lane's rows
+    static constexpr int ROWS = LPH == 1 ? 9 : 3;     // of a lane, at most
+    static constexpr int RUNS = 2 * ROWS;
     // FP64: candidates near r_d kept before they are evaluated
     static constexpr int NEAR = sizeof(T) == 4 ? 1 : 32;
     // run: length, first slot | across a face in x << 27 | row << 28
@@ -234,8 +236,9 @@ __device__ __forceinline__ void density_home(
     // the part across the upper one last
     const bool lo_x = geo.periodic[0] && q0 == 0, hi_x = geo.periodic[0] && q0 == geo.nc[0] - 1;
     const int xb0 = max(q0 - 1, 0), xe0 = min(q0 + 1, geo.nc[0] - 1) + 1;
-    constexpr int ROWS = LPH == 1 ? 9 : 3;
-    const int k0 = LPH == 1 ? 0 : (0x7410 >> 4 * sub) & 15, kend = LPH == 1 ? 9 : (0x9741 >> 4 * sub) & 15;
+    constexpr int ROWS = DensitySmem<T, LPH>::ROWS;
+    constexpr uint32_t SPLIT = LPH == 1 ? 0x90u : 0x96410u;
+    const int k0 = (int)(SPLIT >> 4 * sub & 15u), kend = (int)(SPLIT >> 4 * (sub + 1) & 15u);
     int nrun = 0;
     auto build_runs = [&]() {
         uint32_t b[ROWS], e[ROWS];
@@ -316,6 +319,7 @@ __device__ __forceinline__ void density_home(
     uint32_t nhit = 0, pool = 0;
     bool fits = true;
     for (int pass = 0; pass < (LPH == 1 ? 1 : 2); ++pass) {
+    if (LPH > 1 && pass == 1 && sub == 0) break;
     build_runs();
     // place of mask k: the runs' done ones, before them (LPH > 1) the never used ones
     auto place = [&](int k) {
@@ -383,11 +387,12 @@ __device__ __forceinline__ void density_home(
             uint32_t all = 0;
 #pragma unroll
             for (int t = 0; t < LPH; ++t) {
-                const uint32_t nt = __shfl_sync(group, npass, t, LPH);
+                const uint32_t nt = t == 0 ? 0u : __shfl_sync(group, npass, t, LPH);
                 pool += t < sub ? nt : 0u;
                 all += nt;
             }
-            fits = __all_sync(group, all <= (uint32_t)DN_POOL && run == nrun && len == 0u);
+            fits = __all_sync(group, all <= (uint32_t)DN_POOL &&
+                                         (sub == 0 || (run == nrun && len == 0u)));
         }
         if (nw == 0) break;
 
@@ -411,7 +416,7 @@ __device__ __forceinline__ void density_home(
         };
         auto append = [&](uint32_t j, int code) {
             const uint32_t entry = j << 5 | (uint32_t)code;   // (bits above the slot shift out)
-            if (LPH > 1 && pass == 0) {
+            if (LPH > 1 && pass == 0 && sub != 0) {
                 if (fits) sm.hit[tid / LPH][pool + nhit] = entry;
                 ++nhit;
                 return;
@@ -524,23 +529,28 @@ __device__ __forceinline__ void density_home(
     }
     if constexpr (LPH > 1) {
         if (pass == 1) break;
-        uint32_t all = 0;
+        uint32_t all = 0, before = 0;
+        T sum = T(0);
 #pragma unroll
         for (int t = 0; t < LPH; ++t) {
-            const uint32_t ht = __shfl_sync(group, nhit, t, LPH);
-            acc = rho_add(acc, __shfl_sync(group, part, t, LPH));
-            cnt += t < sub ? ht : 0u;
+            const uint32_t ht = __shfl_sync(group, sub == 0 ? cnt : nhit, t, LPH);
+            sum = rho_add(sum, __shfl_sync(group, part, t, LPH));
+            before += t < sub ? ht : 0u;
             all += ht;
         }
+        acc = sum;
         // wall density: the lanes' sums in a fixed order
         if (WANT_PHI)
 #pragma unroll
             for (int o = 1; o < LPH; o <<= 1) phi += __shfl_xor_sync(group, phi, o);
         if (LIST && fits)
             for (uint32_t k = 0; k < nhit; ++k)
-                if (cnt + k < (uint32_t)NL_MAX)
-                    lp[(int64_t)(cnt + k) * cap] = sm.hit[tid / LPH][pool + k];
-        lp += (int64_t)cnt * cap;
+                if (before + k < (uint32_t)NL_MAX)
+                    lp[(int64_t)(before + k) * cap] = sm.hit[tid / LPH][pool + k];
+        if (sub != 0) {
+            cnt = before;
+            lp += (int64_t)before * cap;
+        }
         pool = all;                            // the home's hits
         if (!LIST || fits || all == 0u) break;
     }

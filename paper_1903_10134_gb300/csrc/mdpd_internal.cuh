@@ -56,9 +56,9 @@ inline double inside_bound(double lo, double hi)
 // blocks x 32 homes, for then a home's chain of instructions is the pass's time.
 // Density pass with one lane a home, with four, and that of a warp per cell which these
 // replaced, us: 1,000 particles 25 / 16 / 20, 8,000 27 / 17 / 20, 20,000 27 / 19 / 22,
-// 30,000 27 / 22 / 24, 38,000 28 / 25 / 26, 40,000 28 / 29 / 26, 80,000 33 / 46 / 41; a
+// 30,000 27 / 21 / 24, 38,000 28 / 23 / 26, 40,000 28 / 29 / 26, 80,000 33 / 46 / 41; a
 // slit of 38,000 with a collapsed liquid, whose dense homes are the pass, 58 / 39 / 33.
-// (FP64: the terms of the middle row, half of them, are one lane's, and four lanes take
+// (Two lanes: 22 to 29 us from 1,000 to 50,000, never the best by more than 2.  FP64: the terms of the middle row, half of them, are one lane's, and four lanes take
 // longer at every size.)
 inline bool density_groups(int64_t homes) { return homes <= 152 * 8 * 32; }
 
