@@ -425,7 +425,7 @@ void set_rho_groups(mdpd_handle* h)
         }
         // (blocks that work in rounds have one lane for a home)
         const bool rounds = ph.frozen && frozen_rounds(all) > 1;
-        ph.rho_groups = density_groups(mobile) && !rounds ? 1 : 0;
+        ph.rho_groups = density_groups(h->precision, mobile) && !rounds ? 1 : 0;
     }
 }
 
@@ -542,7 +542,7 @@ int step_launches(const mdpd_handle* h)
 bool use_split(const mdpd_handle* h)
 {
     return !h->nrep && h->ph.frozen != 0 && !h->ph.list_all &&
-           (h->precision == 0 || !density_groups(h->n)) &&
+           (h->precision == 0 || !density_groups(1, h->n)) &&
            (h->want_phi || h->kernels != MDPD_KERNELS_SCAN);
 }
 

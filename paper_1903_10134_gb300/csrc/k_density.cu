@@ -161,7 +161,7 @@ struct DensitySmem {
     static constexpr int ROWS = LPH == 1 ? 9 : 3;     // of a lane, at most
     static constexpr int RUNS = 2 * ROWS;
     // FP64: candidates near r_d kept before they are evaluated
-    static constexpr int NEAR = sizeof(T) == 4 ? 1 : 32;
+    static constexpr int NEAR = sizeof(T) == 4 ? 1 : LPH == 1 ? 32 : 16;
     // run: length, first slot | across a face in x << 27 | row << 28
     // mask: candidates from the top bit, first slot | across << 27 | row << 28
     uint32_t a[RUNS][PAIR_BLOCK];
@@ -479,6 +479,7 @@ __device__ __forceinline__ void density_home(
                 const uint32_t j = entry >> 5;
                 const T r2 = r2_of(j, (int)(entry & 31u));
                 if (r2 < dc.rc2) {
+                    if (FOLD && ph.rho_groups) fold((entry & 31u) * 11u >> 5 << 28);
                     const T wr = max(T(1) - sqrt_fast(r2) * dc.inv_rd, T(0));
                     const T term = rho_term(dc.cw_rho, wr);      // r = 0 gives w(0)
                     part = rho_add(part, term);
@@ -518,7 +519,7 @@ __device__ __forceinline__ void density_home(
                     in = q < dc.rc2 && q > T(0);
                 }
                 if (mobile && in) append(jr, code);
-                if (!(r2 >= near2) || (want_phi && ((ph.frozen >> (bits & 7u)) & 1u))) {
+                if (pass == 0 && (!(r2 >= near2) || (want_phi && ((ph.frozen >> (bits & 7u)) & 1u)))) {
                     sm.near[nnear++][tid] = entry;
                     if (nnear == DensitySmem<T, LPH>::NEAR) evaluate_near();
                 }
@@ -603,7 +604,7 @@ k_density_nl(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
     static_assert(FS == 0 || !BATCH, "the frozen split is for single systems");
     __shared__ DensitySmem<T, LPH> sm;
     constexpr int HOMES = PAIR_BLOCK / LPH;    // homes of a round
-    constexpr bool FOLD = BATCH && LPH == 1 && sizeof(T) == 4;
+    constexpr bool FOLD = BATCH && LPH == 1;
     pdl_enter();
     if constexpr (FS == 1) {
         // the mobile homes of R * PAIR_BLOCK slots, in slot order (LPH blocks share
@@ -687,10 +688,10 @@ static void density_t(cudaStream_t st, int n, int64_t cap, const Geo& geo, const
         return;
     }
     const bool phi = ph.phi_out != nullptr;
-    const int lph = sizeof(T) == 4 && R == 1 && ph.rho_groups ? 4 : 1;
+    const int lph = R == 1 && ph.rho_groups ? 4 : 1;
     auto k = fs == 1 ? (phi ? k_density_nl<T, false, true, 1, 1, R> : k_density_nl<T, false, false, 1, 1, R>)
                      : (phi ? k_density_nl<T, false, true, 0, 1, 1> : k_density_nl<T, false, false, 0, 1, 1>);
-    if constexpr (sizeof(T) == 4 && R == 1)
+    if constexpr (R == 1)
         if (lph == 4)
             k = fs == 1 ? (phi ? k_density_nl<T, false, true, 1, 4, R> : k_density_nl<T, false, false, 1, 4, R>)
                         : (phi ? k_density_nl<T, false, true, 0, 4, 1> : k_density_nl<T, false, false, 0, 4, 1>);
@@ -740,8 +741,10 @@ void launch_density_only(cudaStream_t st, int precision, int n, const Geo& geo, 
                    start, (T*)nullptr, (uint32_t*)nullptr, (uint32_t*)nullptr,
                    (unsigned long long*)nullptr, src, out);
     };
-    if (precision == 0) go(double{}, k_density_nl<double, false, false, 3, 1, 1>, 1);
-    else if (density_groups(n)) go(float{}, k_density_nl<float, false, false, 3, 4, 1>, 4);
+    const bool shared = density_groups(precision, n);
+    if (precision == 0 && shared) go(double{}, k_density_nl<double, false, false, 3, 4, 1>, 4);
+    else if (precision == 0) go(double{}, k_density_nl<double, false, false, 3, 1, 1>, 1);
+    else if (shared) go(float{}, k_density_nl<float, false, false, 3, 4, 1>, 4);
     else go(float{}, k_density_nl<float, false, false, 3, 1, 1>, 1);
 }
 
@@ -751,9 +754,9 @@ void launch_density_nl_batch(cudaStream_t st, int precision, int64_t cap, const 
                              uint32_t* nl_count)
 {
     if (bt.nchunk <= 0) return;
-    auto f = precision == 0 ? density_batch_t<double, 1>
-             : density_groups((int64_t)bt.nchunk * PAIR_BLOCK) ? density_batch_t<float, 4>
-                                                               : density_batch_t<float, 1>;
+    const bool shared = density_groups(precision, (int64_t)bt.nchunk * PAIR_BLOCK);
+    auto f = precision == 0 ? (shared ? density_batch_t<double, 4> : density_batch_t<double, 1>)
+                            : (shared ? density_batch_t<float, 4> : density_batch_t<float, 1>);
     f(st, cap, bt, pos4, fpos, hpos, cell_s, start, rho, nl, nl_count);
 }
 

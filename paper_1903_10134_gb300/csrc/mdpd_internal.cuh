@@ -51,16 +51,21 @@ inline double inside_bound(double lo, double hi)
     return in > lo ? in : lo;
 }
 
-// Whether the FP32 density pass of a system with this many mobile particles gives each
-// home four lanes (k_density.cu): as long as they fit the chip at once, 152 SMs x 8
-// blocks x 32 homes, for then a home's chain of instructions is the pass's time.
-// Density pass with one lane a home, with four, and that of a warp per cell which these
-// replaced, us: 1,000 particles 25 / 16 / 20, 8,000 27 / 17 / 20, 20,000 27 / 19 / 22,
-// 30,000 27 / 21 / 24, 38,000 28 / 23 / 26, 40,000 28 / 29 / 26, 80,000 33 / 46 / 41; a
-// slit of 38,000 with a collapsed liquid, whose dense homes are the pass, 58 / 39 / 33.
-// (Two lanes: 22 to 29 us from 1,000 to 50,000, never the best by more than 2.  FP64: the terms of the middle row, half of them, are one lane's, and four lanes take
-// longer at every size.)
-inline bool density_groups(int64_t homes) { return homes <= 152 * 8 * 32; }
+// Whether the density pass of a system with this many mobile particles gives each home
+// four lanes (k_density.cu).  In FP32 as long as they fit the chip at once, 152 SMs x 8
+// blocks x 32 homes, for then a home's chain of instructions is the pass's time; in FP64,
+// whose unit four lanes keep busier with the same work, up to 2 blocks per SM.  Density
+// pass with one lane a home, with four, and that of a warp per cell which these replaced,
+// us: FP32 1,000 particles 25 / 16 / 20, 8,000 27 / 17 / 20, 20,000 27 / 19 / 22, 30,000
+// 27 / 21 / 24, 38,000 28 / 23 / 26, 40,000 28 / 29 / 26, 80,000 33 / 46 / 41; a slit of
+// 38,000 with a collapsed liquid, whose dense homes are the pass, 58 / 39 / 33.  FP64, one
+// lane and four: 1,000 45 / 29, 6,000 54 / 37, 10,000 45 / 43, 16,000 46 / 54, 30,000
+// 55 / 96.  (Two lanes, FP32: 22 to 29 us from 1,000 to 50,000, never the best by more
+// than 2.)
+inline bool density_groups(int precision, int64_t homes)
+{
+    return homes <= 152 * 32 * (precision == 0 ? 2 : 8);
+}
 
 // Constants derived from Phys and Geo in the precision of the pair
 // arithmetic, computed once on the host (FP64 arithmetic runs at a small
