@@ -201,6 +201,8 @@ __global__ void k_gather_abar(int n, const uint32_t* __restrict__ id, const doub
 // Bound by issue (FP32: about 130 instructions a pair, 45 of them the draw) and, in
 // FP64, by the FP64 pipe (70 a pair).  The parameters' sums per pair stay out of it:
 // tables in the pair precision, running sums in Sum2.
+// VJP of 100,000 particles in FP32, with the density passes: 624 -> 294 us (FP64 sums,
+// thirteen quotients and gathers of abar by id per pair before).
 template <typename T, bool BATCH>
 __global__ void __launch_bounds__(PAIR_BLOCK)
 k_force_vjp(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,

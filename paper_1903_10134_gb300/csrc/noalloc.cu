@@ -209,7 +209,8 @@ __global__ void k_na_gather(int n, const double* __restrict__ pos, const uint32_
         bool done = sizeof(T) == 4 && cell_offset_f32(x, q[k], f.h[k], f.h_lo[k], f.c0[k], f.c0_lo[k], &o);
         off[k] = (T)o;
         if (__any_sync(__activemask(), !done)) {
-            if (!done) off[k] = to_t<T>(x - fma((double)q[k], geo.h[k], ph.dd.c0[k]));
+            // (one rounding beside that of x - lo: the centre is not rounded)
+            if (!done) off[k] = to_t<T>(fma(-((double)q[k] + 0.5), geo.h[k], x - geo.lo[k]));
         }
         fo[k] = to_f32(off[k]);
     }
