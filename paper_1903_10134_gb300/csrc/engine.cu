@@ -77,6 +77,9 @@ struct mdpd_handle {
     void* rho_ff = nullptr;
     unsigned long long* facc = nullptr;  // cap fixed-point density sums of the frozen split
     bool ff_dirty = true;
+    // the masters were loaded in id order since the last binning: the cell-ordered
+    // arrays still hold the order of the state before
+    bool order_stale = false;
     // positions (by id, n x 3) the frozen-frozen part was computed from, and a
     // device word that set_state raises when a loaded frozen position differs
     double* ffx = nullptr;
@@ -523,6 +526,7 @@ void enqueue_bin(mdpd_handle* h, bool gather_a, bool kick = false)
                            master(h, h->cur), master(h, 1 - h->cur), gather_a, h->geo, h->ph,
                            h->pos4, h->vel4, h->fpos, h->hpos, h->cell_s);
     h->cur = 1 - h->cur;
+    h->order_stale = false;
 }
 
 bool use_split(const mdpd_handle* h);
@@ -546,11 +550,14 @@ bool use_split(const mdpd_handle* h)
            (h->want_phi || h->kernels != MDPD_KERNELS_SCAN);
 }
 
-// The frozen-frozen density part, from the last binning (the frozen
-// particles have not moved since), when the split needs it and it is stale.
+// The frozen-frozen density part, when the split needs it and it is stale, from the
+// last binning (the frozen particles have not moved since).  A state loaded without an
+// evaluation has not been binned yet: a binning, the accelerations gathered along,
+// gives it its cell order first.
 void ensure_ff(mdpd_handle* h)
 {
     if (!use_split(h) || !h->ff_dirty) return;
+    if (h->order_stale) enqueue_bin(h, true);
     launch_density_nl(h->stream, h->precision, (int)h->n, h->cap, h->geo, h->ph, h->pos4, h->fpos,
                       h->hpos, h->cell_s, h->start, h->rho, h->nl, h->nl_count, 2, h->facc, h->id[h->cur],
                       h->rho_ff);
@@ -771,6 +778,7 @@ int run_step(mdpd_handle* h, ForceMode mode, bool kick)
             CK(cudaGraphExecEventRecordNodeSetEvent(gg.exec, gg.ev_node[k], evs[k]));
     CK(cudaGraphLaunch(gg.exec, h->stream));
     h->cur = 1 - h->cur;
+    h->order_stale = false;
     return MDPD_OK;
 }
 
@@ -1418,6 +1426,7 @@ static int set_state_impl(mdpd_handle* h, const double* pos, const double* vel, 
     else
         launch_load_state(st, n, h->cap, d_pos, d_vel, d_acc, h->geo, master(h, c), h->type_by_id,
                           h->status);
+    h->order_stale = true;
     // the frozen-frozen density part stays valid if no frozen particle moved
     // (a caller that resumes or steps a state it read back loads the walls
     // unchanged): compared bit for bit with the positions it came from
@@ -1433,12 +1442,7 @@ static int set_state_impl(mdpd_handle* h, const double* pos, const double* vel, 
         h->ff_dirty = true;
     }
     if (acc) {
-        // no evaluation; when the frozen-frozen part must be recomputed, a
-        // binning (the accelerations gathered along) gives it its cell order
-        if (use_split(h) && h->ff_dirty) {
-            enqueue_bin(h, true);
-            ensure_ff(h);
-        }
+        ensure_ff(h);                         // no evaluation
         CK(cudaGetLastError());
     } else if ((rc = evaluate(h, nullptr, false))) {
         return rc;
@@ -1754,6 +1758,7 @@ void load_state_dev(mdpd_handle* h, const double* pos, const double* vel)
     else
         launch_load_state(h->stream, (int)h->n, h->cap, pos, vel, nullptr, h->geo,
                           master(h, h->cur), h->type_by_id, h->status);
+    h->order_stale = true;
     h->ff_dirty = true;
 }
 
