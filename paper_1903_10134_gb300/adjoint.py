@@ -37,7 +37,7 @@ def _set_tables(system, params, A, B, G):
     each to the host, for all replicas of a batch)."""
     tabs = [t.detach().double().cpu().numpy() for t in (A, B, G)]
     if _is_batch(system):
-        M.mdpd_batch_set_params(system.h, params, [t[:len(params)] for t in tabs])
+        M.mdpd_batch_set_params(system.h, params, tabs)
     else:
         q = params.copy()
         q.A, q.B, q.gamma = (t.copy() for t in tabs)

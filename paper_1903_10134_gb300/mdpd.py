@@ -102,10 +102,13 @@ def to_c_params(p) -> Params:
 
 
 def _c_params_list(params_list, tables=None):
-    """Array of ``mdpd_params``; `tables` = (A, B, gamma), each (len, 8, 8), in
-    place of the objects' own."""
-    cps = (Params * len(params_list))()
-    if not len(params_list):
+    """Array of ``mdpd_params``; `tables` = (A, B, gamma), each one 8 x 8 table per
+    entry of the list, in place of the objects' own."""
+    n = len(params_list)
+    if tables is not None:
+        tables = [_table_stack(t, n, name) for name, t in zip(_TABLES, tables)]
+    cps = (Params * n)()
+    if not n:
         return cps
     view = np.frombuffer(cps, dtype=_PARAMS_DTYPE)      # writes go to cps
     for r, p in enumerate(params_list):
@@ -117,6 +120,16 @@ def _c_params_list(params_list, tables=None):
         for name, t in zip(_TABLES, tables):
             view[name][:] = t
     return cps
+
+
+def _table_stack(t, n, name) -> np.ndarray:
+    """The 8 x 8 corners of the first n tables of `t` (table, type, type).  Anything
+    else is refused: an assignment would broadcast it over replicas or rows."""
+    t = np.asarray(t, dtype=np.float64)
+    if t.ndim != 3 or t.shape[0] < n or min(t.shape[1:]) < MAX_TYPES:
+        raise ValueError(f"{name}: one {MAX_TYPES} x {MAX_TYPES} table per replica is needed "
+                         f"({n} replicas), got shape {t.shape}")
+    return t[:n, :MAX_TYPES, :MAX_TYPES]
 
 
 SYMBOLS = (
@@ -290,7 +303,8 @@ def mdpd_batch_observables(h, mean: bool = False, reset: bool = False) -> np.nda
 
 
 def mdpd_batch_set_params(h, params_list, tables=None):
-    """`tables` = (A, B, gamma), each (nrep, 8, 8), in place of the objects' own."""
+    """`tables` = (A, B, gamma), each (nrep, 8, 8), in place of the objects' own
+    (ValueError for any other shape)."""
     cps = _c_params_list(params_list, tables)
     _check(lib().mdpd_batch_set_params(h, cps), h)
 
