@@ -109,8 +109,10 @@ int mdpd_create_dev(const mdpd_params* params, int64_t n, const double* pos,
  * replica the random stream is keyed on the particle's index inside the
  * replica, so replica r evolves bit-identically to mdpd_create() of
  * (params[r], n[r] particles, seeds[r]) run alone with the same kernel
- * variant.  Walls and the wall density are not available on a batch handle;
- * the VJPs and windows are, with per-replica parameter gradients.
+ * variant (under MDPD_KERNELS_NLIST_THREAD with frozen types, where a system
+ * alone adds their densities in fixed point, up to rounding).  Walls and the
+ * wall density are not available on a batch handle; the VJPs and windows are,
+ * with per-replica parameter gradients.
  * mdpd_step, mdpd_get_state/set_state(_dev), mdpd_forces(_dev),
  * mdpd_set_step, mdpd_sync, mdpd_pair_count (summed over replicas),
  * mdpd_profile, mdpd_set_option and mdpd_autotune apply to the whole batch;
@@ -245,15 +247,21 @@ int mdpd_pair_count(mdpd_handle* h, int64_t* pairs);
  *                      0: launch kernels one by one.
  *   MDPD_OPT_PROFILE   k > 0: record CUDA events around every kernel class of
  *                      the next steps (up to k steps); 0: off.
- *   MDPD_OPT_KERNELS   MDPD_KERNELS_NLIST (default) and
- *                      MDPD_KERNELS_NLIST_THREAD (the same): the density pass
+ *   MDPD_OPT_KERNELS   MDPD_KERNELS_NLIST (default): the density pass
  *                      records each mobile particle's partners within r_c and
- *                      the force pass walks that list; MDPD_KERNELS_SCAN:
- *                      both passes scan the 27 neighbour cells directly.
- *                      Same results up to FP summation order.
+ *                      the force pass walks that list;
+ *                      MDPD_KERNELS_NLIST_THREAD: the same, and in a system
+ *                      with frozen particles the density pass runs for the
+ *                      mobile ones only, which add their terms to the frozen
+ *                      ones' densities in fixed point (frozen split; not on a
+ *                      batch, and not in FP32 up to 38,912 particles);
+ *                      MDPD_KERNELS_SCAN: both passes scan the 27 neighbour
+ *                      cells directly.  Same results up to FP summation order.
  *   MDPD_OPT_WALL_DENSITY  1: every density pass also accumulates the wall
  *                      density phi of each mobile particle (Sec. 3.2,
- *                      Algorithm 1 step 2; read with mdpd_get_wall_density).
+ *                      Algorithm 1 step 2; read with mdpd_get_wall_density);
+ *                      the frozen split is used as under
+ *                      MDPD_KERNELS_NLIST_THREAD while it is on.
  *                      0 (default): off.
  *   MDPD_OPT_FORCE_LANES  1, 2 or 4 (default 1): lanes that share one
  *                      particle's partner list in the force pass (more warps
@@ -374,13 +382,15 @@ int mdpd_window_vjp_dev(mdpd_handle* h, const double* xbar, const double* vbar,
                         const double* cvir, const double* rhobar, double* x0bar, double* v0bar,
                         double* theta_bar);
 
-/* Time the density pass and then the force pass at 1, 2 and 4 lanes per particle
- * (MDPD_OPT_FORCE_LANES; 1 only on a batch) on the current state, reps launches
- * each, and keep the fastest.  The trajectory is not advanced.  A handle on
- * MDPD_KERNELS_SCAN changes to MDPD_KERNELS_NLIST.  chosen (may be NULL, 3
- * ints) receives the density variant, the lanes per particle and 0; ms (may be
- * NULL, 5 doubles) the mean time of the density pass (twice), then of the force
- * pass at 1, 2, 4 lanes (-1: not tried).  Synchronises. */
+/* Time the density pass under MDPD_KERNELS_NLIST and MDPD_KERNELS_NLIST_THREAD
+ * (once where they are the same pass: the variant is then kept, and a handle on
+ * MDPD_KERNELS_SCAN changes to MDPD_KERNELS_NLIST) and then the force pass at 1,
+ * 2 and 4 lanes per particle (MDPD_OPT_FORCE_LANES; 1 only on a batch) on the
+ * current state, reps launches each, and keep the fastest of each.  The
+ * trajectory is not advanced.  chosen (may be NULL, 3 ints) receives the density
+ * variant, the lanes per particle and 0; ms (may be NULL, 5 doubles) the mean
+ * time of the density pass in the two variants, then of the force pass at 1, 2,
+ * 4 lanes (-1: not tried).  Synchronises. */
 int mdpd_autotune(mdpd_handle* h, int32_t reps, int32_t* chosen, double* ms);
 
 /* Grid of the cell lattice (cells per axis) and the kernel launches one step

@@ -539,16 +539,23 @@ int step_launches(const mdpd_handle* h)
 }
 
 // The density pass of a system with frozen particles scans for its mobile homes
-// only (frozen split).  Not in FP32 where all homes fit the chip at once
-// (density_groups): the second kernel costs 4 us there and the homes left out gain
-// nothing.  Density with the split and without, us: rocks of 13,900 / 27,300 / 61,000
-// particles 21 / 25 / 29 and 18 / 21 / 33, slits of 8,200 / 32,800 21 / 26 and 18 / 22.
-bool use_split(const mdpd_handle* h)
+// only (frozen split): under MDPD_KERNELS_NLIST_THREAD, which the caller or the
+// autotuner chooses, and with the wall density, which a batch does not have.  Wall
+// densities are then sums in fixed point (Derived::fix_scale); in FP64 these have a
+// few bits less than FP64 sums, and a replica of a batch, which never splits, must
+// equal its system under MDPD_KERNELS_NLIST to the bit.  Not in FP32 where all homes
+// fit the chip at once (density_groups): the second kernel costs 4 us there and the
+// homes left out gain nothing.  Step with the split and without, us: FP32 rocks of
+// 69,600 / 133,300 / 544,700 / 4,358,100 particles 59 / 85 / 221 / 1,168 and 66 / 86 /
+// 232 / 1,400, slits of 57,600 / 528,000 63 / 292 and 60 / 266; FP64 rocks of 8,800 /
+// 69,600 / 229,700 115 / 243 / 618 and 109 / 250 / 657.
+bool splits(const mdpd_handle* h, int kernels)
 {
     return !h->nrep && h->ph.frozen != 0 && !h->ph.list_all &&
            (h->precision == 0 || !density_groups(1, h->n)) &&
-           (h->want_phi || h->kernels != MDPD_KERNELS_SCAN);
+           (h->want_phi || kernels == MDPD_KERNELS_NLIST_THREAD);
 }
+bool use_split(const mdpd_handle* h) { return splits(h, h->kernels); }
 
 // The frozen-frozen density part, when the split needs it and it is stale, from the
 // last binning (the frozen particles have not moved since).  A state loaded without an
@@ -1964,16 +1971,26 @@ int mdpd_autotune(mdpd_handle* h, int32_t reps, int32_t* chosen, double* ms)
         cudaEventDestroy(e1);
         return code ? h->fail(code, std::string("autotune: ") + what) : MDPD_OK;
     };
-    // 1) the density pass (one variant writes lists; timed for the report)
+    // 1) the density pass of the two list variants, where they differ (frozen split);
+    //    otherwise one timing stands for both and the variant is kept
     LaunchScope scope(step_carveout(h));
     enqueue_bin(h, true);                     // same positions: same order, state kept
-    const int best = h->kernels == MDPD_KERNELS_NLIST_THREAD ? h->kernels : MDPD_KERNELS_NLIST;
-    h->kernels = best;
-    ensure_ff(h);
-    {
-        const double t = time_it([&] { enqueue_density(h); });
-        if (t < 0) return done(MDPD_ERR_CUDA, cudaGetErrorString(cudaGetLastError()));
-        if (ms) ms[0] = ms[1] = t;
+    if (h->kernels == MDPD_KERNELS_SCAN) h->kernels = MDPD_KERNELS_NLIST;
+    const int variants[2] = { MDPD_KERNELS_NLIST, MDPD_KERNELS_NLIST_THREAD };
+    const bool differ = splits(h, variants[0]) != splits(h, variants[1]);
+    double td[2];
+    for (int v = 0; v < (differ ? 2 : 1); ++v) {
+        if (differ) h->kernels = variants[v];
+        ensure_ff(h);
+        td[v] = time_it([&] { enqueue_density(h); });
+        if (td[v] < 0) return done(MDPD_ERR_CUDA, cudaGetErrorString(cudaGetLastError()));
+    }
+    if (!differ) td[1] = td[0];
+    if (td[0] < td[1]) h->kernels = variants[0];
+    const int best = h->kernels;
+    if (ms) {
+        ms[0] = td[0];
+        ms[1] = td[1];
     }
     // 2) lanes per particle of the force pass (evaluation only: the state is kept)
     const int lanes[3] = { 1, 2, 4 };

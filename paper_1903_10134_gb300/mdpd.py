@@ -490,9 +490,9 @@ def mdpd_window_vjp_dev(h, xbar_t=None, vbar_t=None, cvir_t=None, rhobar_t=None,
 
 class Tuned(tuple):
     """Result of mdpd_autotune: unpacks as (density variant, [ms of the density
-    pass, twice]); .lanes is the force pass's lanes per particle, .force_ms its
-    times at 1, 2, 4 lanes (-1: not tried), .shape is 0 (the density pass has one
-    code shape)."""
+    pass under NLIST, NLIST_THREAD]); .lanes is the force pass's lanes per
+    particle, .force_ms its times at 1, 2, 4 lanes (-1: not tried), .shape is 0
+    (the density pass has one code shape)."""
 
     def __new__(cls, chosen, ms):
         t = super().__new__(cls, (int(chosen[0]), [float(x) for x in ms[:2]]))
@@ -503,8 +503,8 @@ class Tuned(tuple):
 
 
 def mdpd_autotune(h, reps: int = 5) -> Tuned:
-    """Time the density pass and pick the fastest lanes per particle of the
-    force pass, on the current state."""
+    """Pick the faster density-pass variant, then the fastest lanes per
+    particle of the force pass, on the current state."""
     chosen = np.zeros(3, np.int32)
     ms = np.zeros(5)
     _check(lib().mdpd_autotune(h, int(reps), _p(chosen), _p(ms)), h)
