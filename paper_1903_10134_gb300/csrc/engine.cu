@@ -102,7 +102,7 @@ struct mdpd_handle {
     int force_lpp = 1;               // lanes per particle of the force pass (single system)
     bool walls_set = false;
     std::vector<int32_t> h_type;
-    std::vector<std::array<int64_t, 8>> type_count;   // particles by type (of each replica)
+    std::array<int64_t, 8> type_count{};   // particles by type (single system)
     int64_t steps_host = 0;
 
     // graphs[profiled][mode: 0 fused, 1 last][cur][first half-kick in the binning]
@@ -415,21 +415,21 @@ void make_geo_phys(const mdpd_params& p, uint64_t seed, Geo& g, Phys& f)
     fill_derived(f, g);
 }
 
-// Phys::rho_groups of the system, or of each replica, from its mobile particles (once
-// the types are known).
+// Phys::rho_groups of each replica: all its particles are homes of its density pass.
+// (A single system's is set with each pass, whose homes may be the mobile ones only.)
 void set_rho_groups(mdpd_handle* h)
 {
-    for (size_t r = 0; r < h->type_count.size(); ++r) {
-        Phys& ph = h->nrep ? h->reps[r].ph : h->ph;
-        int64_t mobile = 0, all = 0;
-        for (int t = 0; t < 8; ++t) {
-            all += h->type_count[r][t];
-            if (!((ph.frozen >> t) & 1u)) mobile += h->type_count[r][t];
-        }
-        // (blocks that work in rounds have one lane for a home)
-        const bool rounds = ph.frozen && frozen_rounds(all) > 1;
-        ph.rho_groups = density_groups(h->precision, mobile) && !rounds ? 1 : 0;
-    }
+    for (int r = 0; r < h->nrep; ++r)
+        h->reps[r].ph.rho_groups = density_groups(h->precision, h->reps[r].n) ? 1 : 0;
+}
+
+// Mobile particles of a single system.
+int64_t num_mobile(const mdpd_handle* h)
+{
+    int64_t m = 0;
+    for (int t = 0; t < 8; ++t)
+        if (!((h->ph.frozen >> t) & 1u)) m += h->type_count[t];
+    return m;
 }
 
 void setup_geo_phys(mdpd_handle* h)
@@ -440,7 +440,6 @@ void setup_geo_phys(mdpd_handle* h)
     make_geo_phys(h->p, h->seed, h->geo, h->ph);
     h->ph.list_all = list_all;
     h->ph.dbg_status = h->status;
-    set_rho_groups(h);
 }
 
 int status_to_code(uint32_t st)
@@ -590,6 +589,9 @@ void enqueue_density(mdpd_handle* h, bool all = false)
     }
     h->ph.phi_out = h->want_phi ? h->phi : nullptr;
     h->ph.list_compact = list_compact(h) ? 1 : 0;
+    // the split's homes are the mobile particles; any other pass's, the adjoint's with
+    // the lists of all particles too, are all of them
+    h->ph.rho_groups = density_groups(h->precision, use_split(h) ? num_mobile(h) : h->n) ? 1 : 0;
     if (h->kernels != MDPD_KERNELS_SCAN || h->want_phi)
         // (the wall density is accumulated by the list pass only)
         launch_density_nl(h->stream, h->precision, (int)h->n, h->cap, h->geo, h->ph, h->pos4,
@@ -861,10 +863,8 @@ int init_handle(mdpd_handle* h, const double* pos, const double* vel, const int3
                     return bail(MDPD_ERR_INVALID_ARG);
                 }
     }
-    h->type_count.assign(bounds.size() - 1, {});
-    for (size_t r = 0; r + 1 < bounds.size(); ++r)
-        for (int64_t i = bounds[r]; i < bounds[r + 1]; ++i) ++h->type_count[r][h->h_type[i]];
-    set_rho_groups(h);
+    if (!h->nrep)
+        for (int32_t t : h->h_type) ++h->type_count[t];
     if ((rc = alloc_particles(h, n))) return bail(rc);
     const int64_t nb = scan_num_blocks(h->geo.ncell);
     if ((rc = dalloc(h, &h->count, (size_t)h->geo.ncell * sizeof(uint32_t))) ||
@@ -1032,6 +1032,7 @@ int create_batch(int32_t nrep, const mdpd_params* params, const int64_t* n, cons
             chunks.push_back(make_int4(r, (int)f, (int)std::min<int64_t>(BATCH_CHUNK, bounds[r + 1] - f), 0));
         wr[r].y = (int)chunks.size() * PAIR_BLOCK_WARPS;
     }
+    set_rho_groups(h);
     h->geo = h->reps[0].geo;
     h->geo.ncell = cells;                  // the concatenated lattice (scan and cell sort)
     h->ph = h->reps[0].ph;
@@ -1268,9 +1269,8 @@ int mdpd_set_walls(mdpd_handle* h, const uint8_t* solid, int32_t nx, int32_t ny,
         return h->fail(MDPD_ERR_CUDA, "wall emission failed");
     }
     h->n = n_new;
-    h->type_count[0][wall_type] += n_new - (int64_t)h->h_type.size();
+    h->type_count[wall_type] += n_new - (int64_t)h->h_type.size();
     h->h_type.resize((size_t)n_new, wall_type);
-    set_rho_groups(h);
     dfree(h->mask_bits);
     h->mask_bits = bits;
     h->mk.bits = bits;

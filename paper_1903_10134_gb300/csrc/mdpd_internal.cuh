@@ -51,8 +51,8 @@ inline double inside_bound(double lo, double hi)
     return in > lo ? in : lo;
 }
 
-// Whether the density pass of a system with this many mobile particles gives each home
-// four lanes (k_density.cu).  In FP32 as long as they fit the chip at once, 152 SMs x 8
+// Whether a density pass over this many homes (all particles, or the mobile ones of the
+// frozen split) gives each four lanes (k_density.cu).  In FP32 as long as they fit the chip at once, 152 SMs x 8
 // blocks x 32 homes, for then a home's chain of instructions is the pass's time; in FP64,
 // whose unit four lanes keep busier with the same work, up to 2 blocks per SM.  Density
 // pass with one lane a home, with four, and that of a warp per cell which these replaced,
