@@ -38,6 +38,7 @@
 // blocks in a fixed order.  Each unordered pair is seen from both sides, so each
 // side adds half its term.
 #include "pair.cuh"
+#include "roots.cuh"
 
 namespace mdpd {
 
@@ -47,21 +48,11 @@ constexpr int TB = 3 * 64;         // parameter slots [q][a][b], q = A, B, gamma
 constexpr int TCOL = 3 * 8;        // per-thread columns [q][partner type]
 
 // 1 / sqrt(x): FP32 from the hardware estimate (2 ulp) with one Newton step, FP64 by
-// the library function.  (Quotients by r are products with it: an FP64 division is
-// some ten instructions at 1/64 of the FP32 rate, and a pair had up to thirteen.)
-__device__ __forceinline__ float inv_sqrt(float x)
-{
-    const float y = rsqrtf(x);
-    return fmaf(0.5f * y, fmaf(-x * y, y, 1.0f), y);
-}
+// the library function (1 ulp; 1 / sqrt has up to 1.5).  (Quotients by r are products
+// with it: an FP64 division is some ten instructions at 1/64 of the FP32 rate, and a
+// pair had up to thirteen.)
+__device__ __forceinline__ float inv_sqrt(float x) { return inv_sqrt_step(x, rsqrtf(x)); }
 __device__ __forceinline__ double inv_sqrt(double x) { return rsqrt(x); }
-// sqrt(x) from y = inv_sqrt(x): in FP32 with the rounding of x y taken back.
-__device__ __forceinline__ float sqrt_from(float x, float y)
-{
-    const float r = x * y;
-    return fmaf(0.5f * y, fmaf(-r, r, x), r);
-}
-__device__ __forceinline__ double sqrt_from(double x, double y) { return x * y; }
 
 // A parameter gradient's running sum over one particle's pairs.  In FP32 a pair of
 // floats (the rounding of every addition kept: Knuth's two-sum), as exact as the
