@@ -55,8 +55,8 @@ __device__ __forceinline__ float inv_sqrt(float x) { return inv_sqrt_step(x, rsq
 __device__ __forceinline__ double inv_sqrt(double x) { return rsqrt(x); }
 
 // A parameter gradient's running sum over one particle's pairs.  In FP32 a pair of
-// floats (the rounding of every addition kept: Knuth's two-sum), as exact as the
-// FP64 sum and off the FP64 pipe.
+// floats (the rounding of every addition kept: Knuth's two-sum): the gradients' errors
+// are those of FP64 sums of the same terms to three digits, off the FP64 pipe.
 struct Sum2 {
     float hi, lo;
 };
@@ -72,6 +72,41 @@ __device__ __forceinline__ void col_add(Sum2& c, float x)
 __device__ __forceinline__ void col_add(double& c, double x) { c += x; }
 __device__ __forceinline__ double col_value(const Sum2& c) { return (double)c.hi + (double)c.lo; }
 __device__ __forceinline__ double col_value(double c) { return c; }
+
+// d(sigma)/d(gamma) of a type pair: in FP64 over sqrt(dt); in FP32 a pair of floats, for
+// every term of the random force's share in the gamma gradient has it as a factor, so
+// its rounding would not average out.
+template <typename T> struct DSigma;
+template <> struct DSigma<float> {
+    using type = float2;
+    static __device__ __forceinline__ float2 make(double d, double)
+    {
+        const float hi = (float)d;
+        return make_float2(hi, (float)(d - (double)hi));
+    }
+};
+template <> struct DSigma<double> {
+    using type = double;
+    static __device__ __forceinline__ double make(double d, double inv_sqrt_dt) { return d * inv_sqrt_dt; }
+};
+// Adds a pair's share hq wc (d xi / sqrt(dt) - wc w) of the gamma gradient, in FP32 with
+// the roundings of the products by hq, wc and d kept (a fused multiply-add gives a
+// product's rounding exactly).
+__device__ __forceinline__ void col_add_gamma(Sum2& col, float hq, float2 d, float wc, float xi,
+                                              float inv_sqrt_dt, float w)
+{
+    const float v = xi * inv_sqrt_dt;
+    const float h = __fmul_rn(hq, wc), he = fmaf(hq, wc, -h);
+    const float m = fmaf(d.x, v, -(wc * w));
+    const float p = __fmul_rn(h, m), pe = fmaf(h, m, -p);
+    col_add(col, p);
+    col.lo = __fadd_rn(col.lo, fmaf(h, d.y * v, fmaf(he, m, pe)));
+}
+__device__ __forceinline__ void col_add_gamma(double& col, double hq, double d, double wc, double xi,
+                                              double, double w)
+{
+    col += hq * wc * (d * xi - wc * w);
+}
 
 // Adjoints of the accelerations in cell order (zero for frozen particles): 16 bytes a
 // slot in FP32, 24 in FP64.
@@ -212,7 +247,7 @@ k_force_vjp(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
     __shared__ Col col[TCOL][PAIR_BLOCK];
     __shared__ T shift[27][3];
     __shared__ PairTables<T> tab;              // A, B, gamma, sigma / sqrt(dt)
-    __shared__ T dsig[64];                     // d(sigma)/d(gamma) / sqrt(dt)
+    __shared__ typename DSigma<T>::type dsig[64];
     __shared__ double wsum[PAIR_BLOCK / 32];
     const BlockSite<BATCH> b = block_site<BATCH>(n, bt);
     const Phys& ph = BATCH ? b.rp->ph : ph_p;             // scalars (and tables if single)
@@ -226,7 +261,8 @@ k_force_vjp(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
         for (int t = 0; t < nt; ++t) col[q * 8 + t][tid] = Col{};
     for (int k = tid; k < 64; k += PAIR_BLOCK) {
         tab.P[k] = make4((T)tabs.A[k], (T)tabs.B[k], (T)tabs.gamma[k], (T)tabs.sigma[k] * dc.inv_sqrt_dt);
-        dsig[k] = tabs.gamma[k] > 0.0 ? (T)(ph.kT / tabs.sigma[k]) * dc.inv_sqrt_dt : T(0);
+        dsig[k] = DSigma<T>::make(tabs.gamma[k] > 0.0 ? ph.kT / tabs.sigma[k] : 0.0,
+                                  ph.dd.inv_sqrt_dt);
     }
     if (tid < 27) {
         shift[tid][0] = (T)(tid % 3 - 1) * dc.h[0];
@@ -317,7 +353,7 @@ k_force_vjp(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
                 const T hq = T(0.5) * qe;
                 col_add(col[tj][tid], hq * wc);
                 col_add(col[8 + tj][tid], hq * rsum * wd);
-                col_add(col[16 + tj][tid], hq * wc * (dsig[pidx] * xi - wc * w));
+                col_add_gamma(col[16 + tj][tid], hq, dsig[pidx], wc, xi, dc.inv_sqrt_dt, w);
             }
             if (vir) {
                 const T mm = T((mob_i ? 1 : 0) + (mob_j ? 1 : 0));
