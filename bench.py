@@ -267,6 +267,13 @@ def candidate_tests(x, params, ncell, frozen=None) -> int:
     return int((cm * neigh).sum())
 
 
+def density_splits(params, n, thread) -> bool:
+    """Whether the density pass of a single system of n particles runs the frozen
+    split: under the nlist-thread variant (`thread`) with frozen types, in FP32 only
+    above the size at which all homes fit the chip at once."""
+    return bool(thread and params.frozen_types and (params.precision == 0 or n > 38912))
+
+
 OBS_NAMES = ("px", "py", "pz", "ke", "kT", "Wxx", "Wyy", "Wzz", "Wxy", "Wxz", "Wyz",
              "sum_vx2", "sum_vy2", "sum_vz2")
 
@@ -645,17 +652,16 @@ def run_ours(args):
         import numpy as np
         xs, _, ts, _ = s.state()
         ws = w if args.workload == "batch" else [w]
-        split_density = args.kernels != "scan"
+        thread = (chosen == mdpd.KERNELS_NLIST_THREAD if tuned
+                  else args.kernels == "nlist-thread")
         off = 0
         cand = 0
         for wr in ws:
             nr = wr.n if args.workload == "batch" else n
             p = wr.params
             ncell = [max(1, int(math.floor(p.box[k] / p.rc))) for k in range(3)]
-            # the list pass of a single system with frozen particles runs the
-            # frozen split
             fz = None
-            if args.workload != "batch" and p.frozen_types and split_density:
+            if args.workload != "batch" and density_splits(p, n, thread):
                 fz = np.isin(ts[off:off + nr], np.array(p.frozen_types))
             cand += candidate_tests(xs[off:off + nr], p, ncell, fz)
             off += nr
