@@ -91,7 +91,10 @@ template <> struct DSigma<double> {
 };
 // Adds a pair's share hq wc (d xi / sqrt(dt) - wc w) of the gamma gradient, in FP32 with
 // the roundings of the products by hq, wc and d kept (a fused multiply-add gives a
-// product's rounding exactly).
+// product's rounding exactly).  Error of the gradient against 64 bits, rms over 300
+// draws, with FP64 terms and sums / one rounded FP32 term a pair / so: liquids of 1,503
+// particles 1.71 / 1.92 / 1.70e-7, of 40,009 1.60 / 1.77 / 1.65e-7; VJP of 100,000
+// particles 301 us with the rounded term, 304 so (two runs of one side differ by more).
 __device__ __forceinline__ void col_add_gamma(Sum2& col, float hq, float2 d, float wc, float xi,
                                               float inv_sqrt_dt, float w)
 {

@@ -573,12 +573,13 @@ __device__ __forceinline__ void density_home(
     if (WANT_PHI) ((T*)ph.phi_out)[s] = phi;
 }
 
-// Frozen split (FS, single systems with frozen particles).  Frozen particles
-// never move, so the part of a frozen particle's density that comes from
-// frozen neighbours is a constant, computed once (k_frozen_part).  FS = 1 then
-// scans for mobile homes only: a mobile home adds each frozen candidate's
-// share w_rho(r_ij) of that candidate's density (the same term it adds to its
-// own) to facc[j] as a fixed-point integer (Derived::fix_scale), by atomic
+// Frozen split (FS, single systems with frozen particles, under
+// MDPD_KERNELS_NLIST_THREAD or with the wall density; the rule and its timings are at
+// engine.cu: splits).  Frozen particles never move, so the part of a frozen particle's
+// density that comes from frozen neighbours is a constant, computed once
+// (k_frozen_part).  FS = 1 then scans for mobile homes only: a mobile home adds each
+// frozen candidate's share w_rho(r_ij) of that candidate's density (the same term it
+// adds to its own) to facc[j] as a fixed-point integer (Derived::fix_scale), by atomic
 // addition, so the sum does not depend on the order; k_frozen_rho then forms
 // rho_j = rho_ff + facc * fix_inv and clears facc.  Each FS = 1 block gathers
 // the mobile homes of R * PAIR_BLOCK slots (R = frozen_rounds) and runs them in
@@ -586,11 +587,12 @@ __device__ __forceinline__ void density_home(
 // (NaN where src has its top bit set).  FS = 0: every particle is
 // a home, and partner lists are written for mobile ones (all under list_all).
 //
-// Bound by issue (82 % of the cycles, L1 data path 70 %): per 32 homes 376 instructions
-// for the runs, 2,228 in the filter, 2,421 for the hits.  Density pass in FP32 before
-// (each candidate in full by one thread, or a warp per cell) and with the filter, us:
-// slab of 820,000 219 / 141, rock of 256^3 voxels (frozen split) 776 / 480, batch of 256
-// liquids (2.8 million) 710 / 476; small systems at density_groups.
+// Bound by issue (77 % of the cycles on the rock of 256^3 voxels, L1 data path 58 %): per
+// 32 homes of a slab 376 instructions for the runs, 2,228 in the filter, 2,421 for the
+// hits.  Density pass in FP32 before (each candidate in full by one thread, or a warp per
+// cell) and with the filter, us: slab of 820,000 219 / 141, rock of 256^3 voxels (frozen
+// split) 776 / 480, batch of 256 liquids (2.8 million) 710 / 476; small systems at
+// density_groups.
 template <typename T, bool BATCH, bool WANT_PHI, int FS, int LPH, int R>
 __global__ void __launch_bounds__(PAIR_BLOCK, sizeof(T) == 4 ? 8 : 5)
 k_density_nl(int n, int64_t cap, Geo geo_p, Phys ph_p, Batch bt,
